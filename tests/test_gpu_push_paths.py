@@ -1,0 +1,64 @@
+"""The push paths of the bit-parallel region discharge: rounds the graph warp
+runs alone, crowded layers handed to the whole block, BFS layers past the
+masks, and switches between them inside one round, on tiles of every shape.
+
+Each result is compared with Dinic and, bit for bit, with the generic kernel
+(kernel_variant 1), which runs the same rounds vertex by vertex."""
+import numpy as np
+import pytest
+
+from gen import grids
+from gen.grids import GridInstance
+from helpers import assert_parity, gpu_solve, opts
+
+pytestmark = pytest.mark.gpu
+
+
+def _serpentine(X, Y, Z, conn):
+    """One corridor that runs through every voxel of each z layer (capacity 3 along it, 0 across), the source at
+    its start and the sink at its end: one tile's BFS has as many layers as the tile has vertices."""
+    H = len(grids.FWD[conn])
+    n = X * Y * Z
+    cs, ct = np.zeros((Z, Y, X), np.int32), np.zeros((Z, Y, X), np.int32)
+    nl = np.zeros((H, Z, Y, X), np.int32)
+    nl[0, :, :, :X - 1] = 3
+    for y in range(Y - 1):
+        nl[1, :, y, X - 1 if y % 2 == 0 else 0] = 3
+    cs[:, 0, 0] = 7
+    cs[:, Y // 2, X // 2] = 2
+    ct[:, Y - 1, X - 1 if Y % 2 else 0] = 9
+    return GridInstance((X, Y, Z), conn, cs.reshape(n), ct.reshape(n), nl.reshape(H, n))
+
+
+def _crowded(X, Y, Z, conn, step):
+    """Excess everywhere, sinks on every step-th column: layers with many vertices in every row."""
+    inst = grids.random_grid((X, Y, Z), conn, 7, cmax=60, tmax=20, p_zero=0.1)
+    x = np.arange(inst.n) % X
+    cs = np.where(x % step == 0, 0, 5 + inst.cs).astype(np.int32)
+    ct = np.where(x % step == 0, 400, 0).astype(np.int32)
+    return GridInstance(inst.dims, conn, cs, ct, inst.nlink)
+
+
+SHAPES = [((70, 37, 1), 4, (32, 32, 1)), ((64, 64, 1), 8, (32, 32, 1)), ((33, 50, 1), 4, (32, 16, 1)),
+          ((64, 31, 1), 8, (32, 16, 1)), ((128, 40, 1), 4, (64, 32, 1)), ((100, 65, 1), 8, (64, 32, 1)),
+          ((64, 64, 1), 4, (64, 64, 1)), ((65, 130, 1), 8, (64, 64, 1)), ((40, 19, 9), 6, (32, 8, 4)),
+          ((64, 16, 8), 6, (32, 8, 8)), ((33, 9, 10), 6, (32, 4, 4)), ((64, 17, 5), 6, (32, 8, 2)),
+          ((50, 33, 9), 6, (32, 16, 8))]
+
+
+@pytest.mark.parametrize("dims,conn,tile", SHAPES)
+@pytest.mark.parametrize("kind", ["serpentine", "crowded2", "crowded9", "crowded32", "sparse"])
+def test_same_as_generic_and_dinic(dims, conn, tile, kind):
+    if kind == "serpentine":
+        inst = _serpentine(*dims, conn)
+    elif kind == "sparse":
+        inst = grids.random_grid(dims, conn, 3, cmax=4, tmax=300, p_zero=0.6)
+    else:
+        inst = _crowded(*dims, conn, int(kind[7:]))
+    got = gpu_solve(inst, tile=tile)
+    assert_parity(inst, got)
+    ref = gpu_solve(inst, tile=tile, opts=opts(kernel_variant=1))
+    for k in ("res", "tres", "exc", "lab"):
+        assert np.array_equal(got[k], ref[k]), k
+    for k in ("sweeps", "discharges", "rounds", "flow_value"):
+        assert getattr(got["stats"], k) == getattr(ref["stats"], k), k
