@@ -474,12 +474,6 @@ __device__ __forceinline__ void discharge2d_region(const Geom &g, const DevState
             for (int d = 0; d < N; ++d) o.to[d] = 0;
             return;
         }
-        int c[N], rc[N], dl[N];
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-            c[d] = s_cap[d * V + i];
-            rc[d] = s_cap[(d ^ 1) * V + i + off(d)];
-        }
         int e = act ? s_exc[i] : 0;
         bool adm[N];
         if (L - 1 <= LCAP) {
@@ -501,12 +495,16 @@ __device__ __forceinline__ void discharge2d_region(const Geom &g, const DevState
         }
 #pragma unroll
         for (int d = 0; d < N; ++d) {
-            dl[d] = adm[d] ? min(e, c[d]) : 0;
-            e -= dl[d];
-            o.to[d] = __ballot_sync(FULL, dl[d] > 0);
+            const int c = s_cap[d * V + i], dl = adm[d] ? min(e, c) : 0;
+            e -= dl;
+            if (dl > 0) {
+                s_cap[d * V + i] = c - dl;
+                s_cap[(d ^ 1) * V + i + off(d)] += dl;
+                atomicAdd(&s_exc[i + off(d)], dl);
+            }
+            o.to[d] = __ballot_sync(FULL, dl > 0);
         }
-        send(i, c, rc, dl);
-        st_if<0>(act, smem_u32(s_exc + i), e);
+        if (act) s_exc[i] = e;
     };
 
     const int klimit = sa.partial ? (sa.sweep_dev ? *sa.sweep_dev : sa.sweep) : INT_MAX;

@@ -10,18 +10,21 @@
 //     index rho = z * TY + y; every mask holds one 32-bit word per row:
 //     R_d[rho] bit x = [c_f(v -> v + D(d)) > 0] for the six arcs
 //     d = +x, -x, +y, -y, +z, -z, T[rho] = [c_f(v,t) > 0], E[rho] = [e_f(v) > 0];
-//   * warp 0 (the graph warp) runs every BFS and reachability flood on these
-//     masks: lane l holds rows l*RPL .. l*RPL+RPL-1; a step shifts a word for
-//     +-x, takes the neighbouring row for +-y (a shuffle across one lane at
-//     the ends of a lane's rows) and the row TY away for +-z (a shuffle across
-//     TY/RPL lanes); floods close whole x-runs at once (Kogge-Stone fill);
+//   * warp 0 (the graph warp) holds these masks in registers, lane l the rows
+//     l*RPL .. l*RPL+RPL-1, and runs every BFS and reachability flood on them: a
+//     step shifts a word for +-x, takes the neighbouring row for +-y (a shuffle
+//     across one lane at the ends of a lane's rows) and the row TY away for +-z
+//     (a shuffle across TY/RPL lanes); floods close whole x-runs at once
+//     (Kogge-Stone fill);
 //   * every arc leaving the tile ends in its own halo cell (six faces), so the
 //     boundary of T_k is a table over halo cells: hm[h] = d(h) if the arc
 //     into h has residual capacity, else infinity;
-//   * all warps do the per-vertex integer work: staging, the layered push,
-//     rebuilding the masks after a push pass, write-back.
+//   * the graph warp also runs the layered push, a lane per row, unless a layer
+//     has many pushing vertices in one row; those layers are pushed by all warps;
+//   * all warps do the staging, the labels and the write-back.
 #include <climits>
 #include <cstdint>
+#include <utility>
 
 #include "mf_internal.cuh"
 
@@ -66,7 +69,10 @@ struct Cfg3D {
     static constexpr size_t smem = (size_t)(N + 3) * V * 4           // cap, tcap, exc, lab
                                    + (size_t)(N + 4) * NR * 4        // R[N], T, E, inc, vis
                                    + (size_t)(LCAP + 1) * NR * 4     // BFS layers 1..LCAP
-                                   + (size_t)2 * HL * 4 + NR + 64;   // halo labels, hm, dirty rows
+                                   + (size_t)2 * HL * 4 + NR + 16;   // halo labels, hm, dirty rows, padding
+    // after this many passes of the graph warp over a push layer the rest of it
+    // is handed to all warps
+    static constexpr int HEAVY = 8;
     static_assert((NR % 32 == 0 || NR == 16) && TY % RPL == 0 && V % NT == 0 && NT % 32 == 0, "tile/threads mismatch");
 };
 
@@ -124,6 +130,49 @@ __device__ __forceinline__ void halo3_src(int h, int &lx, int &ly, int &lz, int 
     lx = q % TX; ly = q / TX; lz = TZ - 1; d = 4;
 }
 
+// highest set bit of a row word; `other` if there is none
+__device__ __forceinline__ int top_bit3(u32 m, int other) {
+    int x;
+    asm("bfind.u32 %0, %1;" : "=r"(x) : "r"(m));
+    return m ? x : other;
+}
+// Predicated shared-memory store at a constant offset (bytes) from an address,
+// and the planes after the vertex at `a` (the address of its cap[0]) sent dl
+// along arc D; c and rc: the residuals of the arc and of its reverse before.
+// An arc has one writer per step, the excess of its head may have several.
+// (Predicated instructions, and an add that is always executed: as conditions
+// these became branches, see ard_discharge2d.cu.)
+template <int OFF>
+__device__ __forceinline__ void st_if3(bool p, unsigned a, int v) {
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.shared.u32 [%0+%3], %1;\n}\n" ::"r"(a), "r"(v),
+                 "r"((unsigned)p), "n"(OFF)
+                 : "memory");
+}
+template <int TY, int V, int D>
+__device__ __forceinline__ void send_arc3(unsigned a, int c, int rc, int dl) {
+    constexpr int off = D == 0 ? 1 : D == 1 ? -1 : D == 2 ? 32 : D == 3 ? -32 : D == 4 ? 32 * TY : -32 * TY;
+    asm volatile(
+        "{\n .reg .pred q;\n setp.ne.s32 q, %3, 0;\n @q st.shared.u32 [%0+%4], %1;\n @q st.shared.u32 [%0+%5], %2;\n"
+        " red.shared.add.u32 [%0+%6], %3;\n}\n" ::"r"(a),
+        "r"(c - dl), "r"(rc + dl), "r"(dl), "n"(4 * D * V), "n"(4 * ((D ^ 1) * V + off)), "n"(4 * (7 * V + off))
+        : "memory");
+}
+template <int TY, int V, int... D>
+__device__ __forceinline__ void send_arcs3(unsigned a, const int (&c)[sizeof...(D)], const int (&rc)[sizeof...(D)],
+                                           const int (&dl)[sizeof...(D)], std::integer_sequence<int, D...>) {
+    (send_arc3<TY, V, D>(a, c[D], rc[D], dl[D]), ...);
+}
+
+// One region's discharge, organised as in 2D (ard_discharge2d.cu): the graph
+// warp keeps the masks in registers, runs the searches and pushes the layers
+// by itself, a lane per row; crowded layers, labels to write and the end of
+// the stages are commands to all warps.
+// Bound by one region's chain of dependent steps (11-12 rounds of 8 BFS layers
+// and 5-6 push layers per discharge).  By all warps, a row per warp with a
+// block barrier per layer and the masks rebuilt after a round, a push layer took
+// 2100-2400 cycles and a BFS layer 320-350, now 1000 and 95.  Discharge time of a
+// solve: 382 -> 209 ms (512x512x384), 12.4 -> 6.9 ms (128^3), 6.1 -> 3.5 ms
+// (61x75x53).
 template <int TY, int TZ, int NT>
 __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState &st, const SweepArgs &sa,
                                                    const int r, unsigned long long *mbar, unsigned &mphase) {
@@ -131,21 +180,24 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     constexpr int TX = 32, N = 6, V = C::V, NR = C::NR, RPL = C::RPL, NW = C::NW, LCAP = C::LCAP, LZ = C::LZ;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smraw[];
-    int *s_cap = (int *)smraw;              // [N][V] residual of arc i -> i + D(d)
+    // (16 bytes of padding first: the reverse arc of the first cell's -x arc is read unconditionally)
+    int *s_cap = (int *)(smraw + 16);       // [N][V] residual of arc i -> i + D(d)
     int *s_tcap = s_cap + N * V;            // [V]
     int *s_exc = s_tcap + V;                // [V]
     int *s_lab = s_exc + V;                 // [V] region label (deep BFS layers: negative tags)
-    u32 *s_R = (u32 *)(s_lab + V);          // [N][NR] residual masks
+    u32 *s_R = (u32 *)(s_lab + V);          // [N][NR] residual masks (rows rebuilt from the planes)
     u32 *s_T = s_R + N * NR;                // [NR]
     u32 *s_E = s_T + NR;                    // [NR]
-    u32 *s_inc = s_E + NR;                  // [NR]
+    u32 *s_inc = s_E + NR;                  // [NR] vertices that joined the closure
     u32 *s_vis = s_inc + NR;                // [NR] final closure (during Augment rounds: excess received)
     u32 *s_layer = s_vis + NR;              // [LCAP+1][NR]
     int *s_hl = (int *)(s_layer + (LCAP + 1) * NR);  // [HL] labels of B^R
     int *s_hm = s_hl + C::HL;               // [HL] label of the halo cell if its arc is residual, else INT_MAX
-    unsigned char *s_dirty = (unsigned char *)(s_hm + C::HL);  // [NR] rows whose planes changed
-    __shared__ int s_ctl[4];
+    // [NR] rows whose planes changed (2: by the current command's pushes)
+    unsigned char *s_dirty = (unsigned char *)(s_hm + C::HL);
+    __shared__ int s_ctl[5];                // command, its argument, epoch, any augmentation, stage
     __shared__ unsigned long long s_flow;
+    enum { kDone = 0, kLabel = 1, kPush = 2 };
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     // does this lane of the graph warp hold tile rows (all do unless the tile has 16 rows)
@@ -159,43 +211,28 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     const int dinf = g.dinf;
     if (tid == 0) s_flow = 0;
 
-    // voxel index i = rho * TX + x, rho = z * TY + y; plane offset of each arc
+    // voxel index i = rho * TX + x, rho = z * TY + y; plane and row offset of each arc
     auto arc_off = [](int d) -> int {
         return d == 0 ? 1 : d == 1 ? -1 : d == 2 ? TX : d == 3 ? -TX : d == 4 ? TX * TY : -TX * TY;
     };
+    auto row_off = [](int d) -> int { return d < 2 ? 0 : d == 2 ? 1 : d == 3 ? -1 : d == 4 ? TY : -TY; };
     // does arc d from row rho stay in the tile along y / z (x handled by the word shifts)
     auto row_has = [](int d, int rho) -> bool {
         const int y = rho % TY, z = rho / TY;
         return d == 2 ? y < TY - 1 : d == 3 ? y > 0 : d == 4 ? z < TZ - 1 : d == 5 ? z > 0 : true;
     };
-    // with only_round, just the rows the last Augment round changed (s_dirty 2)
-    auto rebuild_masks = [&](bool only_round) {
-        for (int i = tid; i < V; i += NT) {
-            const int rho = i / TX;
-            if (only_round && s_dirty[rho] != 2) continue;  // the same row for the whole warp
+    // masks of tile row rho from the planes (one warp)
+    auto rebuild_row = [&](int rho) {
+        const int i = rho * TX + lane;
+        unsigned b[N];
 #pragma unroll
-            for (int d = 0; d < N; ++d) {
-                const unsigned b = __ballot_sync(FULL, s_cap[d * V + i] > 0);
-                if (lane == 0) s_R[d * NR + rho] = b;
-            }
-            const unsigned bt = __ballot_sync(FULL, s_tcap[i] > 0);
-            const unsigned be = __ballot_sync(FULL, s_exc[i] > 0);
-            if (lane == 0) {
-                s_T[rho] = bt;
-                s_E[rho] = be;
-            }
-        }
-    };
-    // with only_round, just the cells whose row the last Augment round changed
-    // (a boundary arc's residual changes only by a push of its own cell)
-    auto rebuild_hm = [&](bool only_round) {
-        for (int h = tid; h < C::HL; h += NT) {
-            int lx, ly, lz, d;
-            halo3_src<TY, TZ>(h, lx, ly, lz, d);
-            const int rho = lz * TY + ly;
-            if (only_round && s_dirty[rho] != 2) continue;
-            const int i = rho * TX + lx;
-            s_hm[h] = s_cap[d * V + i] > 0 ? s_hl[h] : INT_MAX;
+        for (int d = 0; d < N; ++d) b[d] = __ballot_sync(FULL, s_cap[d * V + i] > 0);
+        const unsigned bt = __ballot_sync(FULL, s_tcap[i] > 0), be = __ballot_sync(FULL, s_exc[i] > 0);
+        if (lane == 0) {
+#pragma unroll
+            for (int d = 0; d < N; ++d) s_R[d * NR + rho] = b[d];
+            s_T[rho] = bt;
+            s_E[rho] = be;
         }
     };
 
@@ -249,12 +286,30 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
         }
     }
     __syncthreads();
-    rebuild_masks(false);
-    rebuild_hm(false);
+    for (int rho = warp; rho < NR; rho += NW) rebuild_row(rho);
+    for (int h = tid; h < C::HL; h += NT) {
+        int lx, ly, lz, d;
+        halo3_src<TY, TZ>(h, lx, ly, lz, d);
+        s_hm[h] = s_cap[d * V + (lz * TY + ly) * TX + lx] > 0 ? s_hl[h] : INT_MAX;
+    }
     __syncthreads();
     DIAG_LAP(0);
 
-    // ---- graph-warp helpers (warp 0) ------------------------------------------
+    // ---- the graph warp's state and searches -----------------------------------
+    // (Rm holds no arcs that leave the tile in y or z; those that leave it in x
+    // meet no bit in a shifted word)
+    u32 Rm[N][RPL], T[RPL], E[RPL], Cl[RPL], sdB[RPL];
+    u32 recv[RPL];  // vertices that received excess in this round's push
+#pragma unroll
+    for (int j = 0; j < RPL; ++j) {
+        const int rho = lane * RPL + j;
+#pragma unroll
+        for (int d = 0; d < N; ++d) Rm[d][j] = warp == 0 && lrow && row_has(d, rho) ? s_R[d * NR + rho] : 0;
+        T[j] = warp == 0 && lrow ? s_T[rho] : 0;
+        E[j] = warp == 0 && lrow ? s_E[rho] : 0;
+        Cl[j] = sdB[j] = recv[j] = 0;
+    }
+    bool pushed[RPL] = {};  // rows that pushed
     auto next_stage = [&](int k) -> int {
         int best = INT_MAX;
         for (int h = lane; h < C::HL; h += 32) {
@@ -263,75 +318,87 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
         }
         return __reduce_min_sync(FULL, best);
     };
-    // seed rows of T_k: residual arc to t, or to a halo cell w with d(w) < k
-    auto seed_rows = [&](int k, u32 (&sd)[RPL]) {
+    // boundary part of the seed rows of T_k: a residual arc to a halo cell w with d(w) < k
+    auto seed_boundary = [&](int k) {
 #pragma unroll
         for (int j = 0; j < RPL; ++j) {
             const int rho = lane * RPL + j;
             u32 s = 0u;
             if (lrow) {
-                s = s_T[rho];
                 if (s_hm[C::B_MX + rho] < k) s |= 1u;
                 if (s_hm[C::B_PX + rho] < k) s |= 1u << (TX - 1);
             }
-            sd[j] = s;
+            sdB[j] = s;
         }
+#pragma unroll
         for (int z = 0; z < TZ; ++z) {
             const u32 bm = __ballot_sync(FULL, s_hm[C::B_MY + z * TX + lane] < k);
             const u32 bp = __ballot_sync(FULL, s_hm[C::B_PY + z * TX + lane] < k);
 #pragma unroll
             for (int j = 0; j < RPL; ++j) {
                 const int rho = lane * RPL + j;
-                if (rho == z * TY) sd[j] |= bm;
-                if (rho == z * TY + TY - 1) sd[j] |= bp;
+                if (rho == z * TY) sdB[j] |= bm;
+                if (rho == z * TY + TY - 1) sdB[j] |= bp;
             }
         }
+#pragma unroll
         for (int y = 0; y < TY; ++y) {
             const u32 bm = __ballot_sync(FULL, s_hm[C::B_MZ + y * TX + lane] < k);
             const u32 bp = __ballot_sync(FULL, s_hm[C::B_PZ + y * TX + lane] < k);
 #pragma unroll
             for (int j = 0; j < RPL; ++j) {
                 const int rho = lane * RPL + j;
-                if (rho == y) sd[j] |= bm;
-                if (rho == (TZ - 1) * TY + y) sd[j] |= bp;
+                if (rho == y) sdB[j] |= bm;
+                if (rho == (TZ - 1) * TY + y) sdB[j] |= bp;
             }
         }
     };
-    auto load_masks = [&](u32 (&Rm)[N][RPL]) {
-#pragma unroll
-        for (int j = 0; j < RPL; ++j)
-#pragma unroll
-            for (int d = 0; d < N; ++d) Rm[d][j] = lrow ? s_R[d * NR + lane * RPL + j] : 0u;
-    };
-    // one backward BFS step: vertices with a residual arc into f
-    auto expand = [&](const u32 (&Rm)[N][RPL], const u32 (&f)[RPL], u32 (&out)[RPL]) {
+    // the words of the rows one step along each arc direction (2..5) from the
+    // lane's rows; wrong where the row lies outside the tile (masked by row_has)
+    struct Beside { u32 yp[RPL], ym[RPL], zp[RPL], zm[RPL]; };
+    auto beside = [&](const u32 (&f)[RPL]) -> Beside {
+        Beside o;
         const u32 up = __shfl_up_sync(FULL, f[RPL - 1], 1);
         const u32 dn = __shfl_down_sync(FULL, f[0], 1);
 #pragma unroll
         for (int j = 0; j < RPL; ++j) {
-            const int rho = lane * RPL + j, y = rho % TY, z = rho / TY;
-            const u32 zm = __shfl_up_sync(FULL, f[j], LZ);    // row rho - TY
-            const u32 zp = __shfl_down_sync(FULL, f[j], LZ);  // row rho + TY
-            const u32 fa = j == 0 ? up : f[j - 1];            // row rho - 1
-            const u32 fb = j == RPL - 1 ? dn : f[j + 1];      // row rho + 1
-            u32 a = (Rm[0][j] & (f[j] >> 1)) | (Rm[1][j] & (f[j] << 1));
-            if (y < TY - 1) a |= Rm[2][j] & fb;
-            if (y > 0) a |= Rm[3][j] & fa;
-            if (z < TZ - 1) a |= Rm[4][j] & zp;
-            if (z > 0) a |= Rm[5][j] & zm;
-            out[j] = a;
+            o.zm[j] = __shfl_up_sync(FULL, f[j], LZ);
+            o.zp[j] = __shfl_down_sync(FULL, f[j], LZ);
+            o.ym[j] = j == 0 ? up : f[j > 0 ? j - 1 : 0];
+            o.yp[j] = j == RPL - 1 ? dn : f[j + 1 < RPL ? j + 1 : j];
+        }
+        return o;
+    };
+    // one backward BFS step: vertices with a residual arc into f
+    auto expand = [&](const u32 (&f)[RPL], u32 (&out)[RPL]) {
+        const Beside o = beside(f);
+#pragma unroll
+        for (int j = 0; j < RPL; ++j)
+            out[j] = (Rm[0][j] & (f[j] >> 1)) | (Rm[1][j] & (f[j] << 1)) | (Rm[2][j] & o.yp[j]) | (Rm[3][j] & o.ym[j]) |
+                     (Rm[4][j] & o.zp[j]) | (Rm[5][j] & o.zm[j]);
+    };
+    // words sent along the arcs 2..5 by each row, received by the rows they lead
+    // to: f(d, j) is what the lane's row j sends along arc d, take(d, j, m) gets
+    // what arrives at row j along arc d
+    auto along = [&](auto &&f, auto &&take) {
+        const u32 yp = __shfl_up_sync(FULL, f(2, RPL - 1), 1);   // row - 1 sends to this lane's first row
+        const u32 ym = __shfl_down_sync(FULL, f(3, 0), 1);       // row + 1 sends to its last row
+#pragma unroll
+        for (int j = 0; j < RPL; ++j) {
+            const int rho = lane * RPL + j;
+            const u32 zp = __shfl_up_sync(FULL, f(4, j), LZ), zm = __shfl_down_sync(FULL, f(5, j), LZ);
+            take(2, j, row_has(3, rho) ? (j == 0 ? yp : f(2, j > 0 ? j - 1 : 0)) : 0u);
+            take(3, j, row_has(2, rho) ? (j == RPL - 1 ? ym : f(3, j + 1 < RPL ? j + 1 : j)) : 0u);
+            take(4, j, row_has(5, rho) ? zp : 0u);
+            take(5, j, row_has(4, rho) ? zm : 0u);
         }
     };
-    u32 Cl[RPL];
-#pragma unroll
-    for (int j = 0; j < RPL; ++j) Cl[j] = 0;
-    auto flood = [&](const u32 (&sd)[RPL]) {
-        u32 Rm[N][RPL], fr[RPL], inc[RPL];
-        load_masks(Rm);
+    auto flood = [&]() {
+        u32 fr[RPL], inc[RPL];
         bool any = false;
 #pragma unroll
         for (int j = 0; j < RPL; ++j) {
-            const u32 f = row_fill32(sd[j] & ~Cl[j], Rm[0][j] & ~Cl[j], Rm[1][j] & ~Cl[j]);
+            const u32 f = row_fill32((T[j] | sdB[j]) & ~Cl[j], Rm[0][j] & ~Cl[j], Rm[1][j] & ~Cl[j]);
             Cl[j] |= f;
             inc[j] = f;
             fr[j] = f;
@@ -339,7 +406,7 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
         }
         while (__any_sync(FULL, any)) {
             u32 nf[RPL];
-            expand(Rm, fr, nf);
+            expand(fr, nf);
             any = false;
 #pragma unroll
             for (int j = 0; j < RPL; ++j) {
@@ -355,96 +422,210 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
             for (int j = 0; j < RPL; ++j) s_inc[lane * RPL + j] = inc[j];
         }
     };
-    auto closure_meets_excess = [&]() -> bool {
-        bool m = false;
-#pragma unroll
-        for (int j = 0; j < RPL; ++j) m |= lrow && (Cl[j] & s_E[lane * RPL + j]) != 0u;
-        return __any_sync(FULL, m);
-    };
     auto write_labels = [&](int k) {
         for (int rho = warp; rho < NR; rho += NW)
             if ((s_inc[rho] >> lane) & 1u) s_lab[rho * TX + lane] = k;
     };
 
-    const int klimit = sa.partial ? (sa.sweep_dev ? *sa.sweep_dev : sa.sweep) : INT_MAX;
     long long flow_acc = 0;
-    int rounds = 0, stages = 0, epoch = 0;
-    bool err = false, any_aug = false;
-    bool cl_valid = true;
-
-    // ---- ARD stages ------------------------------------------------------------
-    for (int k = 0;;) {
-        DIAG_MARK();
-        if (warp == 0) {
-            DIAG_ADD(2, 1);
-            u32 sd[RPL];
-            seed_rows(k, sd);
-            if (!cl_valid) {
+    // what the vertex at column x of row rho with excess e, in layer 1, sends
+    // into B^R; returns the rest.  seed: has it still a residual arc into T_k's
+    // boundary vertices (s_hm is kept up to date)
+    auto push_out = [&](int x, int rho, int e, int k, bool &seed) -> int {
+        const int ly = rho % TY, lz = rho / TY, i = rho * TX + x;
+        seed = false;
 #pragma unroll
-                for (int j = 0; j < RPL; ++j) Cl[j] = 0;
-                cl_valid = true;
-            }
-            flood(sd);
-            const bool reach = closure_meets_excess();
-            const int kn = next_stage(k);
-            if (lane == 0) {
-                s_ctl[0] = reach;
-                s_ctl[1] = kn;
+        for (int d = 0; d < N; ++d) {
+            const bool in = d == 0 ? x < TX - 1 : d == 1 ? x > 0 : row_has(d, rho);
+            if (in) continue;
+            const int c = s_cap[d * V + i], h = halo3<TY, TZ>(d, x, ly, lz);
+            if (c > 0 && s_hl[h] < k) {
+                const int b = min(e, c);
+                s_cap[d * V + i] = c - b;
+                e -= b;
+                if (b == c) s_hm[h] = INT_MAX;
+                else seed = true;
             }
         }
-        __syncthreads();
-        DIAG_LAP(1);
-        const int reach = s_ctl[0], kn = s_ctl[1];
-        if (!any_aug) write_labels(k);  // labels stay exact until the first augmentation
-        const bool aug = k <= klimit && !err;
-        if (aug) ++stages;
-        if (aug && reach) {
-            any_aug = true;
-            for (int round = 0;; ++round) {
-                if (round >= sa.max_rounds) { err = true; break; }
-                if (++epoch >= 32767) {  // deep-layer tags wrap: clear them
-                    __syncthreads();
-                    for (int i = tid; i < V; i += NT) s_lab[i] = 0;
-                    __syncthreads();
-                    epoch = 1;
+        return e;
+    };
+    // The vertices of BFS layer L in row rho that have excess (bit `act` of this
+    // lane) push it one layer down, to T_k from layer 1.  Returns the vertices
+    // that pushed along each arc; bpush tells of pushes into B^R.
+    struct PushOut { u32 to[N]; bool bpush; };
+    auto push_row = [&](int rho, bool act, int L, int k, int epoch, u32 sd, PushOut &o) {
+        const int x = lane, i = rho * TX + x;
+        o.bpush = false;
+        if (L == 1) {
+            int e = act ? s_exc[i] : 0;
+            const int tc = act ? s_tcap[i] : 0;
+            const int dl = min(e, tc);
+            if (dl > 0) {
+                s_tcap[i] = tc - dl;
+                e -= dl;
+                flow_acc += dl;
+            }
+            o.bpush = (__ballot_sync(FULL, e > 0) & sd) != 0;
+            bool seed;
+            if (o.bpush && e > 0) e = push_out(x, rho, e, k, seed);
+            if (act) s_exc[i] = e;
+#pragma unroll
+            for (int d = 0; d < N; ++d) o.to[d] = 0;
+            return;
+        }
+        bool adm[N];
+        if (L - 1 <= LCAP) {
+            const u32 *lay = s_layer + (L - 1) * NR;
+            const u32 bit = 1u << x, l0 = lay[rho];
+            adm[0] = (l0 & (bit << 1)) != 0;
+            adm[1] = (l0 & (bit >> 1)) != 0;
+#pragma unroll
+            for (int d = 2; d < N; ++d) adm[d] = row_has(d, rho) && (lay[rho + row_off(d)] & bit);
+        } else {
+            const int tg = deep_tag3(epoch, L - 1);
+#pragma unroll
+            for (int d = 0; d < N; ++d) {
+                const bool in = d == 0 ? x < TX - 1 : d == 1 ? x > 0 : row_has(d, rho);
+                adm[d] = in && s_lab[i + arc_off(d)] == tg;
+            }
+        }
+        int e = act ? s_exc[i] : 0;
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            const int c = s_cap[d * V + i];
+            const int dl = adm[d] ? min(e, c) : 0;
+            e -= dl;
+            if (dl > 0) {
+                s_cap[d * V + i] = c - dl;
+                s_cap[(d ^ 1) * V + i + arc_off(d)] += dl;
+                atomicAdd(&s_exc[i + arc_off(d)], dl);
+            }
+            o.to[d] = __ballot_sync(FULL, dl > 0);
+        }
+        if (act) s_exc[i] = e;
+    };
+
+    const int klimit = sa.partial ? (sa.sweep_dev ? *sa.sweep_dev : sa.sweep) : INT_MAX;
+    int rounds = 0, stages = 0, epoch = 0;
+    bool err = false, any_aug = false;
+    bool cl_valid = true;  // Cl is the closure of T_k on the current graph (empty at start)
+
+    // ---- ARD stages: the graph warp decides, all warps execute its commands ------
+    enum { kFlood, kRound, kNext };
+    int phase = kFlood, k = 0, kn = 0, round = 0, resume = 0;
+    for (;;) {
+        if (warp == 0) {
+            int cmd = kDone, arg = 0;
+            for (;;) {
+                if (phase == kFlood) {
+                    DIAG_MARK();
+                    DIAG_ADD(2, 1);
+                    if (!cl_valid) {
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) Cl[j] = 0;
+                        cl_valid = true;
+                    }
+                    seed_boundary(k);
+                    flood();
+                    bool m = false;
+#pragma unroll
+                    for (int j = 0; j < RPL; ++j) m |= (Cl[j] & E[j]) != 0;
+                    const bool reach = __any_sync(FULL, m);
+                    kn = next_stage(k);
+                    const bool aug = k <= klimit && !err;
+                    if (aug) ++stages;
+                    DIAG_LAP(1);
+                    if (aug && reach) {
+                        phase = kRound;
+                        round = 0;
+                        any_aug = true;
+                    } else {
+                        phase = kNext;
+                        if (!any_aug) {  // labels stay exact until the first augmentation
+                            cmd = kLabel;
+                            arg = k;
+                            break;
+                        }
+                    }
+                    continue;
                 }
-                DIAG_MARK();
-                if (warp == 0) {
+                if (phase == kNext) {
+                    // nothing left to learn: labels are recomputed at the end anyway
+                    if (kn == INT_MAX || (any_aug && (kn > klimit || err))) break;
+                    k = kn;
+                    phase = kFlood;
+                    continue;
+                }
+                // a round of Augment(R, T_k): exact BFS + layered push
+                if (resume == 0 && round >= sa.max_rounds) {
+                    err = true;
+                    cl_valid = false;
+                    phase = kNext;
+                    continue;
+                }
+                int L = resume;  // > 0: the block has pushed the layers above
+                resume = 0;
+                if (L == 0) {
+                    if (++epoch >= 32767) {  // deep-layer tags wrap: clear them
+                        for (int i = lane; i < V; i += 32) s_lab[i] = 0;
+                        __syncwarp();
+                        epoch = 1;
+                    }
+                    DIAG_MARK();
                     DIAG_ADD(5, 1);
-                    u32 Rm[N][RPL], vis[RPL], fr[RPL], want[RPL];
-                    load_masks(Rm);
-                    seed_rows(k, fr);
                     int lmax = 0;
+                    u32 vis[RPL], fr[RPL], want[RPL];
                     bool pending = false;
 #pragma unroll
                     for (int j = 0; j < RPL; ++j) {
-                        const int rho = lane * RPL + j;
-                        const u32 ex = lrow ? s_E[rho] & Cl[j] : 0u;  // excess that can reach T_k lies in the closure
-                        vis[j] = fr[j];
-                        if (lrow) {
-                            s_layer[1 * NR + rho] = fr[j];
-                            s_vis[rho] = 0u;  // vertices that receive excess in this round's push
-                        }
+                        const u32 ex = E[j] & Cl[j];  // excess that can reach T_k lies in the closure
+                        recv[j] = 0;
+                        vis[j] = fr[j] = T[j] | sdB[j];
+                        if (lrow) s_layer[1 * NR + lane * RPL + j] = fr[j];
                         if (fr[j] & ex) lmax = 1;
                         want[j] = ex & ~vis[j];
                         pending |= want[j] != 0u;
                     }
-                    int L = 1;
-                    while (__any_sync(FULL, pending)) {
-                        u32 nf[RPL];
-                        expand(Rm, fr, nf);
+                    L = 1;
+                    bool go = __any_sync(FULL, pending);
+                    // two layers per vote: a layer too many is an empty or unused mask
+                    while (go && L + 2 <= LCAP) {
                         bool any = false;
+                        pending = false;
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            u32 nf[RPL];
+                            expand(fr, nf);
+                            ++L;
+#pragma unroll
+                            for (int j = 0; j < RPL; ++j) {
+                                nf[j] &= ~vis[j];
+                                vis[j] |= nf[j];
+                                fr[j] = nf[j];
+                                if (lrow) s_layer[L * NR + lane * RPL + j] = nf[j];
+                                if (nf[j] & want[j]) lmax = L;
+                                want[j] &= ~nf[j];
+                            }
+                        }
 #pragma unroll
                         for (int j = 0; j < RPL; ++j) {
-                            nf[j] &= ~vis[j];
-                            any |= nf[j] != 0u;
+                            any |= fr[j] != 0u;
+                            pending |= want[j] != 0u;
                         }
-                        if (!__any_sync(FULL, any)) break;
+                        const bool a = __any_sync(FULL, any), b = __any_sync(FULL, pending);
+                        go = a && b;
+                    }
+                    while (go) {  // layers past the masks: label tags
+                        u32 nf[RPL];
+                        expand(fr, nf);
                         ++L;
+                        bool any = false;
                         pending = false;
 #pragma unroll
                         for (int j = 0; j < RPL; ++j) {
                             const int rho = lane * RPL + j;
+                            nf[j] &= ~vis[j];
+                            any |= nf[j] != 0u;
                             vis[j] |= nf[j];
                             fr[j] = nf[j];
                             if (L <= LCAP) {
@@ -457,138 +638,279 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
                             want[j] &= ~nf[j];
                             pending |= want[j] != 0u;
                         }
+                        const bool a = __any_sync(FULL, any), b = __any_sync(FULL, pending);
+                        go = a && b;
                     }
-                    lmax = __reduce_max_sync(FULL, lmax);
-                    if (lane == 0) s_ctl[2] = lmax;
                     DIAG_ADD(6, L);
+                    lmax = __reduce_max_sync(FULL, lmax);
+                    __syncwarp();
+                    DIAG_LAP(4);
+                    if (lmax == 0) {  // no excess vertex reaches T_k: stage done
+                        cl_valid = false;
+                        phase = kNext;
+                        continue;
+                    }
+                    ++rounds;
+                    ++round;
+                    DIAG_ADD(8, lmax);
+                    L = lmax;
                 }
-                __syncthreads();
-                DIAG_LAP(4);
-                const int Lmax = s_ctl[2];
-                if (Lmax == 0) break;  // no excess vertex reaches T_k: stage done
-                ++rounds;
                 // layered push, top layer first: layer L pushes only to layer L-1
                 // (to T_k from layer 1), so every arc has one writer per step.
-                // Only vertices that had excess when the round began (s_E) or
-                // received some in an earlier step of it (s_vis) can push, so
-                // rows without such a vertex of layer L are passed over.
-                u32 *s_recv = s_vis;
-                for (int L = Lmax; L >= 1; --L) {
-                    const int tgL = deep_tag3(epoch, L), tgL1 = deep_tag3(epoch, L - 1);
-                    const bool lo_mask = L - 1 <= LCAP;
-                    for (int rho = warp; rho < NR; rho += NW) {
-                        const u32 P = (L <= LCAP ? s_layer[L * NR + rho] : FULL) & (s_E[rho] | s_recv[rho]);
-                        if (!P) continue;
-                        u32 A[N];
-                        if (L > 1 && lo_mask) {
-                            const u32 *lay = s_layer + (L - 1) * NR;
-                            const u32 l0 = lay[rho];
-                            A[0] = s_R[0 * NR + rho] & (l0 >> 1);
-                            A[1] = s_R[1 * NR + rho] & (l0 << 1);
+                // Only vertices that had excess when the round began or received
+                // some in an earlier step of it can push.  A lane takes the
+                // vertices of its own rows one after another.
+                DIAG_MARK();
+                u32 to[N][RPL];  // vertices that pushed along arc d in this round
 #pragma unroll
-                            for (int d = 2; d < N; ++d) {
-                                const int o = d == 2 ? 1 : d == 3 ? -1 : d == 4 ? TY : -TY;
-                                A[d] = row_has(d, rho) ? (s_R[d * NR + rho] & lay[rho + o]) : 0u;
-                            }
-                        }
-                        bool pushed = false;
-                        const int lx = lane, i = rho * TX + lx;
-                        const int ly = rho % TY, lz = rho / TY;
-                        bool act = (P >> lx) & 1u;
-                        if (act && L > LCAP) act = s_lab[i] == tgL;
-                        int e = act ? s_exc[i] : 0;
-                        if (e > 0) {
-                            const int e0 = e;
-                            if (L == 1) {
-                                const int tc = s_tcap[i];
-                                if (tc > 0) {
-                                    const int dl = min(e, tc);
-                                    s_tcap[i] = tc - dl;
-                                    e -= dl;
-                                    flow_acc += dl;
-                                }
+                for (int j = 0; j < RPL; ++j)
 #pragma unroll
-                                for (int d = 0; d < N; ++d) {
-                                    if (e == 0) break;
-                                    const int nx = lx + arc_dx(6, d), ny = ly + arc_dy(6, d), nz = lz + arc_dz(6, d);
-                                    if (nx >= 0 && nx < TX && ny >= 0 && ny < TY && nz >= 0 && nz < TZ) continue;
-                                    const int c = s_cap[d * V + i];
-                                    if (c > 0 && s_hl[halo3<TY, TZ>(d, lx, ly, lz)] < k) {
-                                        const int dl = min(e, c);
-                                        s_cap[d * V + i] = c - dl;
-                                        e -= dl;
-                                    }
-                                }
-                            } else {
+                    for (int d = 0; d < N; ++d) to[d][j] = 0;
+                if (L <= LCAP) {  // (layers without masks are left to the block)
+                    // the lane's words of layers L, L - 1 and L - 2 (loaded a step ahead;
+                    // layer 0 is unused space), and the rows beside of layer L - 1
+                    u32 lw[RPL], lo[RPL], ln[RPL];
+                    auto layer_word = [&](int l, int j) -> u32 { return lrow ? s_layer[l * NR + lane * RPL + j] : 0u; };
 #pragma unroll
-                                for (int d = 0; d < N; ++d) {
-                                    if (e == 0) break;
-                                    const int nx = lx + arc_dx(6, d), ny = ly + arc_dy(6, d), nz = lz + arc_dz(6, d);
-                                    bool adm;
-                                    if (lo_mask) {
-                                        adm = (A[d] >> lx) & 1u;
-                                    } else {
-                                        adm = nx >= 0 && nx < TX && ny >= 0 && ny < TY && nz >= 0 && nz < TZ &&
-                                              s_lab[i + arc_off(d)] == tgL1 && s_cap[d * V + i] > 0;
-                                    }
-                                    if (!adm) continue;
-                                    const int j = i + arc_off(d);
-                                    const int c = s_cap[d * V + i];
-                                    const int dl = min(e, c);
-                                    s_cap[d * V + i] = c - dl;
-                                    s_cap[(d ^ 1) * V + j] += dl;
-                                    atomicAdd(&s_exc[j], dl);
-                                    atomicOr(&s_recv[j >> 5], 1u << (j & 31));
-                                    e -= dl;
-                                }
-                            }
-                            s_exc[i] = e;
-                            pushed = e != e0;
-                        }
-                        if (__any_sync(FULL, pushed) && lane < 5) {
-                            const int o = lane == 0 ? -TY : lane == 1 ? -1 : lane == 2 ? 0 : lane == 3 ? 1 : TY;
-                            const int rr = rho + o;
-                            if (rr >= 0 && rr < NR) s_dirty[rr] = 2;  // changed in this round
-                        }
+                    for (int j = 0; j < RPL; ++j) {
+                        lw[j] = layer_word(L, j);
+                        lo[j] = layer_word(L - 1, j);
                     }
-                    __syncthreads();
+                    Beside bo = beside(lo);
+                    bool heavy = false;
+                    for (; L > 1; --L) {
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) ln[j] = layer_word(L - 2, j);
+                        const Beside bn = beside(ln);
+                        u32 P[RPL];
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) {
+                            P[j] = lw[j] & (E[j] | recv[j]);
+                            pushed[j] |= P[j] != 0u;
+                        }
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) {
+                            const int rho = lane * RPL + j;
+                            u32 src[N];  // bit x: the head of arc d from column x lies in layer L - 1
+                            src[0] = lo[j] >> 1;
+                            src[1] = lo[j] << 1;
+                            src[2] = row_has(2, rho) ? bo.yp[j] : 0u;
+                            src[3] = row_has(3, rho) ? bo.ym[j] : 0u;
+                            src[4] = row_has(4, rho) ? bo.zp[j] : 0u;
+                            src[5] = row_has(5, rho) ? bo.zm[j] : 0u;
+                            int x = top_bit3(P[j], lane);
+                            // no branches inside: lanes without a vertex run along with
+                            // amounts of 0, in a column of their own (no bank conflicts)
+                            for (int it = 0;; ++it) {
+                                const u32 bit = (1u << x) & P[j];
+                                const int i = rho * TX + x;
+                                int c[N], rc[N], dl[N];
+#pragma unroll
+                                for (int d = 0; d < N; ++d) {
+                                    c[d] = s_cap[d * V + i];
+                                    rc[d] = s_cap[(d ^ 1) * V + i + arc_off(d)];
+                                }
+                                int e = s_exc[i];
+                                P[j] ^= bit;
+                                x = top_bit3(P[j], lane);
+                                const bool again = __any_sync(FULL, P[j] != 0u);
+#pragma unroll
+                                for (int d = 0; d < N; ++d) {
+                                    dl[d] = (src[d] & bit) ? min(e, c[d]) : 0;
+                                    e -= dl[d];
+                                }
+                                send_arcs3<TY, V>(smem_u32(s_cap + i), c, rc, dl, std::make_integer_sequence<int, N>());
+#pragma unroll
+                                for (int d = 0; d < N; ++d) {  // (an arc with c = 0 has no bit in Rm)
+                                    if (dl[d] != 0) to[d][j] |= bit;
+                                    if (dl[d] == c[d]) Rm[d][j] &= ~bit;
+                                }
+                                st_if3<4 * (N + 1) * V>(bit != 0u, smem_u32(s_cap + i), e);
+                                E[j] = (E[j] & ~bit) | (e > 0 ? bit : 0u);
+                                if (!again) break;
+                                if (it == C::HEAVY) {  // the rest of a crowded layer is left to the block
+                                    heavy = true;
+                                    break;
+                                }
+                            }
+                        }
+                        // who received (marks of earlier layers are sent again: harmless)
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) recv[j] |= (to[0][j] << 1) | (to[1][j] >> 1);
+                        along([&](int d, int j) { return to[d][j]; }, [&](int, int j, u32 m) { recv[j] |= m; });
+                        __syncwarp();
+                        if (heavy) {  // layer L shrinks to the vertices that have not pushed
+#pragma unroll
+                            for (int j = 0; j < RPL; ++j)
+                                if (lrow) s_layer[L * NR + lane * RPL + j] = P[j];
+                            break;
+                        }
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) {
+                            lw[j] = lo[j];
+                            lo[j] = ln[j];
+                        }
+                        bo = bn;
+                    }
+                    if (!heavy) {
+#pragma unroll
+                        for (int j = 0; j < RPL; ++j) {
+                            const int rho = lane * RPL + j;
+                            u32 P = lw[j] & (E[j] | recv[j]);
+                            pushed[j] |= P != 0u;
+                            int x = top_bit3(P, lane);
+                            for (bool again = true; again;) {
+                                const u32 bit = (1u << x) & P;
+                                const int xv = x, i = rho * TX + x;
+                                int e = bit ? s_exc[i] : 0;
+                                const int tc = s_tcap[i];
+                                P ^= bit;
+                                x = top_bit3(P, lane);
+                                again = __any_sync(FULL, P != 0u);
+                                const int dl = min(e, tc);
+                                e -= dl;
+                                flow_acc += dl;
+                                const bool out = e > 0 && (sdB[j] & bit);
+                                if (__any_sync(FULL, out)) {
+                                    if (out) {
+                                        bool seed;
+                                        e = push_out(xv, rho, e, k, seed);
+                                        if (!seed) sdB[j] &= ~bit;
+                                    }
+                                }
+                                st_if3<4 * N * V>(bit != 0u, smem_u32(s_cap + i), tc - dl);
+                                st_if3<4 * (N + 1) * V>(bit != 0u, smem_u32(s_cap + i), e);
+                                T[j] &= dl == tc ? ~bit : ~0u;
+                                E[j] = (E[j] & ~bit) | (e > 0 ? bit : 0u);
+                            }
+                        }
+                        __syncwarp();
+                        L = 0;
+                    }
                 }
+                // the reverse arcs of the pushes are residual now
+#pragma unroll
+                for (int j = 0; j < RPL; ++j) {
+                    Rm[1][j] |= to[0][j] << 1;
+                    Rm[0][j] |= to[1][j] >> 1;
+                }
+                along([&](int d, int j) { return to[d][j]; }, [&](int d, int j, u32 m) { Rm[d ^ 1][j] |= m; });
                 DIAG_LAP(7);
-                rebuild_masks(true);  // a push changes its row and the rows one step away in y and z only
-                rebuild_hm(true);
-                __syncthreads();
-                for (int rho = tid; rho < NR; rho += NT)
-                    if (s_dirty[rho] == 2) s_dirty[rho] = 1;
-                DIAG_LAP(3);
-                DIAG_ADD(8, Lmax);
+                if (L >= 1) {
+                    cmd = kPush;
+                    arg = L;
+                    break;
+                }
             }
-            if (warp == 0) cl_valid = false;  // the residual graph changed
+            if (cmd == kPush) {
+#pragma unroll
+                for (int j = 0; j < RPL; ++j)
+                    if (lrow) {
+                        s_E[lane * RPL + j] = E[j];
+                        s_vis[lane * RPL + j] = recv[j];
+                        s_inc[lane * RPL + j] = sdB[j];
+                    }
+            }
+            if (lane == 0) {
+                s_ctl[0] = cmd;
+                s_ctl[1] = arg;
+                s_ctl[2] = epoch;
+                s_ctl[3] = any_aug;
+                s_ctl[4] = k;
+            }
         }
-        if (kn == INT_MAX) break;
-        if (any_aug && (kn > klimit || err)) break;
-        k = kn;
         __syncthreads();
+        const int cmd = s_ctl[0], arg = s_ctl[1];
+        if (cmd == kDone) break;
+        if (cmd == kLabel) {
+            write_labels(arg);
+            __syncthreads();
+            continue;
+        }
+        DIAG_MARK();
+        // the push layers from arg down by all warps: warp w takes the busy
+        // rows w, w + NW, .. of each layer, while a layer is crowded
+        const int ep = s_ctl[2], kk = s_ctl[4];
+        u32 *s_recv = s_vis;
+        int L = arg;
+        for (; L >= 1; --L) {
+            u32 mine[RPL];
+            bool many = false;
+            int rank0 = 0;
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                const int rho = lane + 32 * q;
+                u32 P = 0;
+                // (deep layers: every row, as marks of the step itself would show in the word)
+                if (rho < NR) P = L <= LCAP ? s_layer[L * NR + rho] & (s_E[rho] | s_recv[rho]) : FULL;
+                many |= __popc(P) > C::HEAVY / 2;
+                const unsigned busy = __ballot_sync(FULL, P != 0u);
+                const int rank = rank0 + __popc(busy & ((1u << lane) - 1u));
+                mine[q] = __ballot_sync(FULL, P != 0u && rank % NW == warp);
+                rank0 += __popc(busy);
+            }
+            if (!__any_sync(FULL, many)) break;  // (the same in every warp) back to the graph warp
+#pragma unroll
+            for (int q = 0; q < RPL; ++q)
+                for (u32 mm = mine[q]; mm; mm &= mm - 1) {
+                    const int rho = 32 * q + __ffs((int)mm) - 1;
+                    const u32 P = (L <= LCAP ? s_layer[L * NR + rho] : FULL) & (s_E[rho] | s_recv[rho]);
+                    bool act = (P >> lane) & 1u;
+                    if (L > LCAP) act = act && s_lab[rho * TX + lane] == deep_tag3(ep, L);
+                    if (!__any_sync(FULL, act)) continue;
+                    PushOut o;
+                    push_row(rho, act, L, kk, ep, s_inc[rho], o);
+                    if (lane < 5) {  // the row itself and the rows beside
+                        const int d = lane == 0 ? 0 : lane + 1;
+                        const u32 v = lane == 0 ? (o.to[0] << 1) | (o.to[1] >> 1) : lane == 1 ? o.to[2] : lane == 2 ? o.to[3]
+                                                                                  : lane == 3 ? o.to[4] : o.to[5];
+                        if (v) atomicOr(&s_recv[rho + row_off(d)], v);
+                        if (v || lane == 0) s_dirty[rho + row_off(d)] = 2;
+                    }
+                }
+            __syncthreads();
+        }
+        for (int rho = warp; rho < NR; rho += NW)
+            if (s_dirty[rho] == 2) rebuild_row(rho);
+        __syncthreads();
+        if (warp == 0) {
+#pragma unroll
+            for (int j = 0; j < RPL; ++j) {
+                const int rho = lane * RPL + j;
+                if (lrow && s_dirty[rho] == 2) {
+#pragma unroll
+                    for (int d = 0; d < N; ++d) Rm[d][j] = row_has(d, rho) ? s_R[d * NR + rho] : 0u;
+                    T[j] = s_T[rho];
+                    E[j] = s_E[rho];
+                    s_dirty[rho] = 1;
+                }
+                recv[j] = lrow ? s_recv[rho] : 0u;
+            }
+            __syncwarp();
+            seed_boundary(k);
+            resume = L;
+        }
+        DIAG_LAP(13);
     }
 
     // ---- region-relabel after augmentation: d(u) = min{k : u -> T_k} -------------
-    if (any_aug) {
+    if (s_ctl[3]) {
         DIAG_MARK();
-        __syncthreads();
+        __syncthreads();  // the last command has been read
         if (warp == 0) {
 #pragma unroll
             for (int j = 0; j < RPL; ++j) Cl[j] = 0;
         }
         for (int k2 = 0;;) {
             if (warp == 0) {
-                u32 sd[RPL];
-                seed_rows(k2, sd);
-                flood(sd);
+                seed_boundary(k2);
+                flood();
                 const int n2 = next_stage(k2);
-                if (lane == 0) s_ctl[3] = n2;
+                if (lane == 0) s_ctl[0] = n2;
             }
             __syncthreads();
             write_labels(k2);
-            const int n2 = s_ctl[3];
+            const int n2 = s_ctl[0];
             __syncthreads();
             if (n2 == INT_MAX) break;
             k2 = n2;
@@ -597,7 +919,16 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     }
     if (warp == 0 && lrow) {
 #pragma unroll
-        for (int j = 0; j < RPL; ++j) s_vis[lane * RPL + j] = Cl[j];
+        for (int j = 0; j < RPL; ++j) {
+            const int rho = lane * RPL + j;
+            s_vis[rho] = Cl[j];
+            if (pushed[j]) {  // rows to write back: those that pushed and the rows beside
+                s_dirty[rho] = 1;
+#pragma unroll
+                for (int d = 2; d < N; ++d)
+                    if (row_has(d, rho)) s_dirty[rho + row_off(d)] = 1;
+            }
+        }
     }
     __syncthreads();
     DIAG_MARK();
