@@ -10,14 +10,29 @@ import pytest
 from gen import grids
 from gen.grids import GridInstance
 from helpers import assert_parity, gpu_solve, opts
+from paper_1109_1146_gb300.mf import arcs_of
 
 pytestmark = pytest.mark.gpu
+
+
+def _random(dims, conn, seed, **kw):
+    """grids.random_grid, also on the stencils of Sec. 7.1 (links leaving the grid removed)."""
+    if conn < 100:
+        return grids.random_grid(dims, conn, seed, **kw)
+    X, Y, _ = dims
+    base = grids.random_grid(dims, 4, seed, **kw)
+    nl = np.concatenate([grids.random_grid(dims, 4, seed + h, **kw).nlink[:1] for h in range(arcs_of(conn) // 2)])
+    nl = nl.reshape(-1, Y, X)
+    for h, (dx, dy) in enumerate(((1, 0), (0, 1)) + grids.PAPER_DISPLACEMENTS[2:arcs_of(conn) // 2]):
+        nl[h, max(0, Y - dy):, :] = 0
+        nl[h, :, max(0, X - dx):] = 0
+    return GridInstance(dims, conn, base.cs, base.ct, nl.reshape(len(nl), -1))
 
 
 def _serpentine(X, Y, Z, conn):
     """One corridor that runs through every voxel of each z layer (capacity 3 along it, 0 across), the source at
     its start and the sink at its end: one tile's BFS has as many layers as the tile has vertices."""
-    H = len(grids.FWD[conn])
+    H = arcs_of(conn) // 2
     n = X * Y * Z
     cs, ct = np.zeros((Z, Y, X), np.int32), np.zeros((Z, Y, X), np.int32)
     nl = np.zeros((H, Z, Y, X), np.int32)
@@ -32,7 +47,7 @@ def _serpentine(X, Y, Z, conn):
 
 def _crowded(X, Y, Z, conn, step):
     """Excess everywhere, sinks on every step-th column: layers with many vertices in every row."""
-    inst = grids.random_grid((X, Y, Z), conn, 7, cmax=60, tmax=20, p_zero=0.1)
+    inst = _random((X, Y, Z), conn, 7, cmax=60, tmax=20, p_zero=0.1)
     x = np.arange(inst.n) % X
     cs = np.where(x % step == 0, 0, 5 + inst.cs).astype(np.int32)
     ct = np.where(x % step == 0, 400, 0).astype(np.int32)
@@ -43,7 +58,8 @@ SHAPES = [((70, 37, 1), 4, (32, 32, 1)), ((64, 64, 1), 8, (32, 32, 1)), ((33, 50
           ((64, 31, 1), 8, (32, 16, 1)), ((128, 40, 1), 4, (64, 32, 1)), ((100, 65, 1), 8, (64, 32, 1)),
           ((64, 64, 1), 4, (64, 64, 1)), ((65, 130, 1), 8, (64, 64, 1)), ((40, 19, 9), 6, (32, 8, 4)),
           ((64, 16, 8), 6, (32, 8, 8)), ((33, 9, 10), 6, (32, 4, 4)), ((64, 17, 5), 6, (32, 8, 2)),
-          ((50, 33, 9), 6, (32, 16, 8))]
+          ((50, 33, 9), 6, (32, 16, 8)), ((70, 37, 1), 108, (32, 32, 1)), ((64, 64, 1), 112, (32, 32, 1)),
+          ((33, 50, 1), 116, (32, 32, 1)), ((40, 65, 1), 124, (32, 32, 1)), ((67, 40, 1), 128, (32, 32, 1))]
 
 
 @pytest.mark.parametrize("dims,conn,tile", SHAPES)
@@ -52,7 +68,7 @@ def test_same_as_generic_and_dinic(dims, conn, tile, kind):
     if kind == "serpentine":
         inst = _serpentine(*dims, conn)
     elif kind == "sparse":
-        inst = grids.random_grid(dims, conn, 3, cmax=4, tmax=300, p_zero=0.6)
+        inst = _random(dims, conn, 3, cmax=4, tmax=300, p_zero=0.6)
     else:
         inst = _crowded(*dims, conn, int(kind[7:]))
     got = gpu_solve(inst, tile=tile)
