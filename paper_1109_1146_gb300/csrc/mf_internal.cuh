@@ -246,7 +246,7 @@ bool discharge_supported(int conn, int tx, int ty, int tz);
 // the synthetic stencils of Sec. 7.1 (codes 100 + c), generic kernel, single solves;
 // their exact region-distance relabel (glr_stencil.cu, 32x32 tiles)
 bool stencil_glr_supported(int conn, const Geom &g);
-size_t stencil_glr_scratch_bytes(const Geom &g);
+size_t stencil_glr_scratch_bytes(int conn, const Geom &g);
 cudaError_t stencil_glr(int conn, const Geom &g, const DevState &st, void *scratch, cudaStream_t s);
 bool discharge_paper_supported(int conn, int tx, int ty, int tz);
 size_t discharge_paper_smem_bytes(int conn, int tx, int ty, int tz);
