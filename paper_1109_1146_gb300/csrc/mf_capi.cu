@@ -264,25 +264,35 @@ __global__ void validate_batch_kernel(const ValJob *__restrict__ jobs, const int
 
 // A region is "touched" in a sweep when it or one of its neighbour regions
 // (across a stencil arc) was discharged: only those can see their boundary
-// flow, excess or labels change.
+// flow, excess or labels change.  region_flags gathers the discharged flags
+// around region r for a whole warp in one round of loads, a bit per neighbour
+// (3D: across the six faces and the region itself; 2D: the 3 x 3 block, where
+// the 4-connected grid has no arc to the corner regions).
 template <int CONN>
-__device__ __forceinline__ bool region_touched(const Geom &g, const DevState &st, int r) {
-    if (st.disc[r]) return true;
-    const int rx = r % g.RX, ry = (r / g.RX) % g.RY, rz = r / (g.RX * g.RY);
-    if constexpr (is_paper(CONN)) {  // displacements up to 4 < tile width: the eight surrounding regions
-        for (int qy = ry - 1; qy <= ry + 1; ++qy)
-            for (int qx = rx - 1; qx <= rx + 1; ++qx)
-                if (qx >= 0 && qx < g.RX && qy >= 0 && qy < g.RY && st.disc[qy * g.RX + qx]) return true;
-        return false;
+__device__ __forceinline__ int region_bit(int qx, int qy, int qz) {
+    return CONN == 6 ? (qx ? (qx < 0 ? 0 : 1) : qy ? (qy < 0 ? 2 : 3) : qz ? (qz < 0 ? 4 : 5) : 6) : (qy + 1) * 3 + qx + 1;
+}
+template <int CONN> constexpr int kOwnRegion = CONN == 6 ? 6 : 4;
+template <int CONN>
+__device__ __forceinline__ unsigned region_flags(const Geom &g, const DevState &st, int rx, int ry, int rz) {
+    const int lane = threadIdx.x & 31;
+    int qx = 0, qy = 0, qz = 0;
+    bool in = false;
+    if (CONN == 6) {
+        in = lane < 7;
+        qx = lane == 0 ? -1 : lane == 1;
+        qy = lane == 2 ? -1 : lane == 3;
+        qz = lane == 4 ? -1 : lane == 5;
     } else {
-#pragma unroll
-        for (int d = 0; d < arcs_of(CONN); ++d) {
-            const int qx = rx + arc_dx(CONN, d), qy = ry + arc_dy(CONN, d), qz = rz + arc_dz(CONN, d);
-            if (qx < 0 || qx >= g.RX || qy < 0 || qy >= g.RY || qz < 0 || qz >= g.RZ) continue;
-            if (st.disc[(qz * g.RY + qy) * g.RX + qx]) return true;
-        }
-        return false;
+        in = lane < 9 && (CONN != 4 || lane % 2 == 1 || lane == 4);
+        qx = lane % 3 - 1;
+        qy = lane / 3 - 1;
     }
+    qx += rx;
+    qy += ry;
+    qz += rz;
+    in = in && qx >= 0 && qx < g.RX && qy >= 0 && qy < g.RY && qz >= 0 && qz < g.RZ;
+    return __ballot_sync(0xffffffffu, in && st.disc[((size_t)qz * g.RY + qy) * g.RX + qx] != 0);
 }
 
 __device__ __forceinline__ int hist_bin(int l) { return l < kHistBins ? l : kHistBins; }
@@ -294,52 +304,89 @@ __device__ __forceinline__ int hist_bin(int l) { return l < kHistBins ? l : kHis
 //   a refused push goes back to its sender (residual and excess restored).
 // Also commits the new boundary labels and keeps the histogram of boundary
 // labels (Sec. 5.3: the global gap needs labels of B only) up to date.
-// Fusion of one boundary vertex u = (lx, ly, lz) of region r (see above).
-// The boundary-label histogram change is returned as (old bin, new bin), -1
-// where there is none, for the caller to aggregate over its warp.
+// Fusion of one boundary vertex u = (lx, ly, lz) of region r at (rx, ry, rz)
+// (see above).  near: the discharged regions around r (region_flags).  The
+// boundary-label histogram change is returned as (old bin, new bin), -1 where
+// there is none, for the caller to aggregate over its warp.
 template <int CONN>
-__device__ __forceinline__ void fuse_cell(const Geom &g, const DevState &st, const int r, const int lx, const int ly,
-                                          const int lz, const bool discr, int &bin_old, int &bin_new) {
-    const int rx = r % g.RX, ry = (r / g.RX) % g.RY, rz = r / (g.RX * g.RY);
+__device__ __forceinline__ void fuse_cell(const Geom &g, const DevState &st, const int rx, const int ry, const int rz,
+                                          const unsigned near, const int lx, const int ly, const int lz, int &bin_old,
+                                          int &bin_new) {
+    constexpr int N = arcs_of(CONN);
     const size_t n = (size_t)g.n;
     const int x = rx * g.tx + lx, y = ry * g.ty + ly, z = rz * g.tz + lz;
     bin_old = bin_new = -1;
     if (!in_grid(g, x, y, z)) return;
     const size_t u = ((size_t)z * g.Y + y) * g.X + x;
-    bool boundary = false;
-    int back_total = 0;
-    int du = -1;
-#pragma unroll
-    for (int d = 0; d < arcs_of(CONN); ++d) {
+    const bool discr = (near >> kOwnRegion<CONN>) & 1u;
+    // the flow over every crossing arc and u's labels: independent loads, one
+    // round trip (the Sec. 7.1 stencils have too many arcs to hold and take
+    // them one by one below)
+    int pu[is_paper(CONN) ? 1 : N], pw[is_paper(CONN) ? 1 : N];
+    bool boundary = false, flow = false;
+    auto load = [&](int d, int &a, int &b, size_t &w) {
         const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d), wz = z + arc_dz(CONN, d);
-        if (!in_grid(g, wx, wy, wz)) continue;
-        const int rw = region_of(g, wx, wy, wz);
-        if (rw == r) continue;
-        if (!boundary) {
-            boundary = true;
-            du = discr ? st.lab_next[u] : st.lab[u];
+        a = b = 0;
+        w = 0;
+        if (!in_grid(g, wx, wy, wz)) return;
+        const int qx = (wx >> g.sx) - rx, qy = (wy >> g.sy) - ry, qz = (wz >> g.sz) - rz;
+        if (!(qx | qy | qz)) return;
+        boundary = true;
+        w = ((size_t)wz * g.Y + wy) * g.X + wx;
+        if (discr) a = st.bout[(size_t)d * n + u];
+        if ((near >> region_bit<CONN>(qx, qy, qz)) & 1u) b = st.bout[(size_t)(d ^ 1) * n + w];
+    };
+    if constexpr (!is_paper(CONN)) {
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            size_t w;
+            load(d, pu[d], pw[d], w);
         }
-        const size_t w = ((size_t)wz * g.Y + wy) * g.X + wx;
-        const bool discw = st.disc[rw];
-        const int pu = discr ? st.bout[(size_t)d * n + u] : 0;
-        const int pw = discw ? st.bout[(size_t)(d ^ 1) * n + w] : 0;
-        if (!(pu | pw)) continue;  // no flow crossed this arc: nothing to accept or return
-        const int dw = discw ? st.lab_next[w] : st.lab[w];
-        const int back = (dw <= du + 1 ? 0 : pu) + (du <= dw + 1 ? pw : 0);
-        if (back) {
-            st.cap[(size_t)d * n + u] += back;
-            back_total += back;
+    } else {
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d);
+            boundary |= wx >= 0 && wx < g.X && wy >= 0 && wy < g.Y && ((wx >> g.sx) != rx || (wy >> g.sy) != ry);
         }
     }
     if (!boundary) return;
-    if (back_total) st.exc[u] += back_total;
-    if (discr) {
-        const int old = st.lab[u];
-        if (old != du) {
-            if (old < g.dinf) bin_old = hist_bin(old);
-            if (du < g.dinf) bin_new = hist_bin(du);
-            st.lab[u] = du;
+    const int old = st.lab[u];
+    const int du = discr ? st.lab_next[u] : old;
+    if constexpr (!is_paper(CONN)) {
+#pragma unroll
+        for (int d = 0; d < N; ++d) flow |= (pu[d] | pw[d]) != 0;
+    } else {
+        flow = true;
+    }
+    if (flow) {  // else no flow crossed an arc of u: nothing to accept or return
+        int back_total = 0;
+#pragma unroll
+        for (int d = 0; d < N; ++d) {
+            int a, b;
+            if constexpr (is_paper(CONN)) {
+                size_t w;
+                load(d, a, b, w);
+            } else {
+                a = pu[d];
+                b = pw[d];
+            }
+            if (!(a | b)) continue;
+            const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d), wz = z + arc_dz(CONN, d);
+            const size_t w = ((size_t)wz * g.Y + wy) * g.X + wx;
+            const bool discw = (near >> region_bit<CONN>((wx >> g.sx) - rx, (wy >> g.sy) - ry, (wz >> g.sz) - rz)) & 1u;
+            const int dw = discw ? st.lab_next[w] : st.lab[w];
+            const int back = (dw <= du + 1 ? 0 : a) + (du <= dw + 1 ? b : 0);
+            if (back) {
+                st.cap[(size_t)d * n + u] += back;
+                back_total += back;
+            }
         }
+        if (back_total) st.exc[u] += back_total;
+    }
+    if (discr && old != du) {
+        if (old < g.dinf) bin_old = hist_bin(old);
+        if (du < g.dinf) bin_new = hist_bin(du);
+        st.lab[u] = du;
     }
 }
 
@@ -375,8 +422,8 @@ __device__ __forceinline__ void surface_cell(const Geom &g, bool is3d, int p, in
     if (p < 2 * A) {
         lz = p < A ? 0 : g.tz - 1;
         const int q = p < A ? p : p - A;
-        lx = q % g.tx;
-        ly = q / g.tx;
+        lx = q & (g.tx - 1);
+        ly = q >> g.sx;
         return;
     }
     p -= 2 * A;
@@ -384,8 +431,8 @@ __device__ __forceinline__ void surface_cell(const Geom &g, bool is3d, int p, in
     if (p < 2 * Bf) {
         ly = p < Bf ? 0 : g.ty - 1;
         const int q = p < Bf ? p : p - Bf;
-        lx = q % g.tx;
-        lz = 1 + q / g.tx;
+        lx = q & (g.tx - 1);
+        lz = 1 + (q >> g.sx);
         return;
     }
     p -= 2 * Bf;
@@ -396,67 +443,50 @@ __device__ __forceinline__ void surface_cell(const Geom &g, bool is3d, int p, in
     lz = 1 + q / (g.ty - 2);
 }
 
-// region_touched for a whole warp in one round of loads: lane d reads the
-// flag of the neighbour region across arc d (the 3 x 3 block of regions for
-// the Sec. 7.1 stencils), the next lane the region's own
+// Fusion of one touched region over the tile surface (only surface cells can
+// be boundary vertices) by `split` warps, this one taking every split-th chunk
+// of 32 cells; returns whether the region was touched.
 template <int CONN>
-__device__ __forceinline__ bool region_touched_warp(const Geom &g, const DevState &st, int r) {
-    const int lane = threadIdx.x & 31;
+__device__ __forceinline__ bool fuse_region_warp(const Geom &g, const DevState &st, const int r, const int part = 0,
+                                                 const int split = 1) {
     const int rx = r % g.RX, ry = (r / g.RX) % g.RY, rz = r / (g.RX * g.RY);
-    bool f = false;
-    if constexpr (is_paper(CONN)) {
-        if (lane < 9) {
-            const int qx = rx + lane % 3 - 1, qy = ry + lane / 3 - 1;
-            if (qx >= 0 && qx < g.RX && qy >= 0 && qy < g.RY) f = st.disc[qy * g.RX + qx] != 0;
-        }
-    } else {
-        if (lane < CONN) {
-            const int qx = rx + arc_dx(CONN, lane), qy = ry + arc_dy(CONN, lane), qz = rz + arc_dz(CONN, lane);
-            if (qx >= 0 && qx < g.RX && qy >= 0 && qy < g.RY && qz >= 0 && qz < g.RZ)
-                f = st.disc[(qz * g.RY + qy) * g.RX + qx] != 0;
-        } else if (lane == CONN) {
-            f = st.disc[r] != 0;
-        }
-    }
-    return __any_sync(0xffffffffu, f);
-}
-
-// Fusion of one touched region by one warp over the tile surface (only
-// surface cells can be boundary vertices).
-template <int CONN>
-__device__ __forceinline__ void fuse_region_warp(const Geom &g, const DevState &st, const int r) {
-    if (!region_touched_warp<CONN>(g, st, r)) return;
-    const bool discr = st.disc[r];
+    const unsigned near = region_flags<CONN>(g, st, rx, ry, rz);
+    if (!near) return false;
     // boundary vertices lie on the tile surface, or (the longer displacements
     // of Sec. 7.1) anywhere in a band of the stencil's width: all cells then
     const int P = is_paper(CONN) ? g.tx * g.ty : surface_cells(g, CONN == 6);
-    for (int p0 = 0; p0 < P; p0 += 32) {  // whole warp per step: the histogram update is a warp operation
+    for (int p0 = part * 32; p0 < P; p0 += 32 * split) {  // whole warp per step: the histogram update is a warp operation
         const int p = p0 + (threadIdx.x & 31);
         int bo = -1, bn = -1;
         if (p < P) {
             int lx, ly, lz;
             if (is_paper(CONN)) { lx = p & (g.tx - 1); ly = p >> g.sx; lz = 0; }
             else surface_cell(g, CONN == 6, p, lx, ly, lz);
-            fuse_cell<CONN>(g, st, r, lx, ly, lz, discr, bo, bn);
+            fuse_cell<CONN>(g, st, rx, ry, rz, near, lx, ly, lz, bo, bn);
         }
         hist_update_warp(st.hist, bo, bn);
     }
+    return true;
 }
 
 // Activity of one region after the fusion (one warp): with a gap, every label
 // g < d < d_inf of the tile becomes d_inf first (all cells); a touched region
 // is active if its discharge left interior excess (left_active) or a surface
 // vertex has excess below d_inf.
-template <int CONN>
-__device__ __forceinline__ void post_region_warp(const Geom &g, const DevState &st, const int r, const int gap) {
+// (PARTS: of `split` warps, each taking every split-th chunk of 32 cells; the
+// fusion has set active to left_active, a warp that finds an active vertex sets
+// it, and finish_flags_kernel counts)
+template <int CONN, bool PARTS>
+__device__ __forceinline__ void post_region_warp(const Geom &g, const DevState &st, const int r, const int gap,
+                                                 const int part = 0, const int split = 1) {
     const int lane = threadIdx.x & 31;
-    const bool touched = region_touched_warp<CONN>(g, st, r);
-    if (!touched && gap == 0) return;
     const int rx = r % g.RX, ry = (r / g.RX) % g.RY, rz = r / (g.RX * g.RY);
-    int act = touched ? st.left_active[r] : 0;
+    const bool touched = region_flags<CONN>(g, st, rx, ry, rz) != 0;
+    if (!touched && gap == 0) return;
+    int act = touched && !PARTS ? st.left_active[r] : 0;
     if (gap > 0) {
         const int V = g.tx * g.ty * g.tz;
-        for (int i = lane; i < V; i += 32) {
+        for (int i = part * 32 + lane; i < V; i += 32 * split) {
             const int lx = i & (g.tx - 1), ly = (i >> g.sx) & (g.ty - 1), lz = i >> (g.sx + g.sy);
             const int x = rx * g.tx + lx, y = ry * g.ty + ly, z = rz * g.tz + lz;
             if (!in_grid(g, x, y, z)) continue;
@@ -473,7 +503,7 @@ __device__ __forceinline__ void post_region_warp(const Geom &g, const DevState &
         }
     } else {
         const int P = is_paper(CONN) ? g.tx * g.ty : surface_cells(g, CONN == 6);
-        for (int p = lane; p < P && !act; p += 32) {
+        for (int p = part * 32 + lane; p < P && !act; p += 32 * split) {
             int lx, ly, lz;
             if (is_paper(CONN)) { lx = p & (g.tx - 1); ly = p >> g.sx; lz = 0; }
             else surface_cell(g, CONN == 6, p, lx, ly, lz);
@@ -485,24 +515,45 @@ __device__ __forceinline__ void post_region_warp(const Geom &g, const DevState &
     }
     act = __any_sync(0xffffffffu, act);
     if (lane == 0 && touched) {
+        if (PARTS) {
+            if (act) st.active[r] = 1;
+            return;
+        }
         st.active[r] = (unsigned char)act;
         if (act) atomicAdd(&st.ctr[kActiveRegions], 1);
     }
 }
 
-// single 3D grid: a warp per region, grid-stride
-template <int CONN>
-__global__ void fuse_warp_kernel(const Geom g, const DevState st) {
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < g.nreg; r += nw)
-        fuse_region_warp<CONN>(g, st, r);
+// single grid: `split` warps per region, grid-stride.  A region is a chain of
+// dependent loads per chunk of 32 surface cells (4 chunks in a 32x32 tile, 21 in
+// 32x8x4, 32 for the Sec. 7.1 stencils), so a grid with fewer regions than the
+// chip holds warps spreads the chunks over them; with more regions one warp each
+// is cheaper (the test whether a region was touched is made once).
+static int surface_split(const Geom &g, int conn) {
+    const int cells = is_paper(conn) ? g.tx * g.ty
+                      : conn == 6 ? 2 * g.tx * g.ty + 2 * g.tx * (g.tz - 2) + 2 * (g.ty - 2) * (g.tz - 2)
+                                  : 2 * g.tx + 2 * (g.ty - 2);
+    return std::max(1, std::min((cells + 31) / 32, device_sms() * 64 / g.nreg));
 }
 template <int CONN>
-__global__ void post_warp_kernel(const Geom g, const DevState st) {
+__global__ void fuse_warp_kernel(const Geom g, const DevState st, const int split) {
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    const int items = g.nreg * split;  // (split > 1 only below the number of warps the chip holds)
+    for (int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < items; k += nw) {
+        const int r = split == 1 ? k : k / split, part = k - r * split;
+        if (fuse_region_warp<CONN>(g, st, r, part, split) && part == 0 && (threadIdx.x & 31) == 0)
+            st.active[r] = st.left_active[r];
+    }
+}
+template <int CONN>
+__global__ void post_warp_kernel(const Geom g, const DevState st, const int split) {
     const int gap = st.ctr[kGap];
     const int nw = gridDim.x * (blockDim.x >> 5);
-    for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < g.nreg; r += nw)
-        post_region_warp<CONN>(g, st, r, gap);
+    const int items = g.nreg * split;
+    for (int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < items; k += nw) {
+        const int r = split == 1 ? k : k / split;
+        post_region_warp<CONN, true>(g, st, r, gap, k - r * split, split);
+    }
 }
 
 // Global gap (Sec. 5.1, with the boundary-label histogram of Sec. 5.3): the
@@ -531,81 +582,6 @@ __device__ __forceinline__ void gap_find_body(const DevState &st) {
 }
 
 __global__ void gap_find_kernel(const DevState st) { gap_find_body(st); }
-
-// ---- 2D fusion and activity over perimeter items -----------------------------
-// One thread per (region, perimeter slot): only tile perimeters hold boundary
-// vertices, so the 2D sweep kernels walk 2 tx + 2 (ty - 2) slots per region
-// instead of whole tiles (a warp covers one region's perimeter, and its lanes
-// share the region-touched test through the cache).
-__device__ __forceinline__ void perimeter_xy(int p, int tx, int ty, int &lx, int &ly) {
-    if (p < tx) { lx = p; ly = 0; }
-    else if (p < 2 * tx) { lx = p - tx; ly = ty - 1; }
-    else if (p < 2 * tx + ty - 2) { lx = 0; ly = 1 + p - 2 * tx; }
-    else { lx = tx - 1; ly = 1 + p - 2 * tx - (ty - 2); }
-}
-
-__device__ __forceinline__ int perimeter_slots(const Geom &g) { return 2 * g.tx + 2 * (g.ty - 2); }
-
-// Algorithm 2's fusion for one boundary vertex u of region r (gather form;
-// see fuse_region); also restarts the activity of a touched region from the
-// excess its discharge left inside the tile.
-template <int CONN>
-__global__ void fuse2d_kernel(const Geom g, const DevState st) {
-    const int P = perimeter_slots(g);
-    const long long items = (long long)g.nreg * P;
-    const int lane = threadIdx.x & 31;
-    // warp-uniform steps (the histogram update is a warp operation)
-    for (long long k0 = blockIdx.x * (long long)blockDim.x + (threadIdx.x - lane); k0 < items;
-         k0 += (long long)gridDim.x * blockDim.x) {
-        const long long k = k0 + lane;
-        int bo = -1, bn = -1;
-        if (k < items) {
-            const int r = (int)(k / P), p = (int)(k % P);
-            if (region_touched<CONN>(g, st, r)) {
-                if (p == 0) st.active[r] = st.left_active[r];
-                int lx, ly;
-                perimeter_xy(p, g.tx, g.ty, lx, ly);
-                fuse_cell<CONN>(g, st, r, lx, ly, 0, st.disc[r] != 0, bo, bn);
-            }
-        }
-        hist_update_warp(st.hist, bo, bn);
-    }
-}
-
-// Activity after the fusion: a touched region is active if its discharge left
-// interior excess or a perimeter vertex has excess below d_inf.  With a gap,
-// first every label g < d < d_inf in the grid becomes d_inf (all vertices).
-template <int CONN>
-__global__ void post2d_kernel(const Geom g, const DevState st) {
-    const int gap = st.ctr[kGap];
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    if (gap == 0) {
-        const int P = perimeter_slots(g);
-        const long long items = (long long)g.nreg * P;
-        for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < items; k += stride) {
-            const int r = (int)(k / P), p = (int)(k % P);
-            int lx, ly;
-            perimeter_xy(p, g.tx, g.ty, lx, ly);
-            const int x = (r % g.RX) * g.tx + lx, y = (r / g.RX) * g.ty + ly;
-            if (x >= g.X || y >= g.Y) continue;
-            const size_t u = (size_t)y * g.X + x;
-            if (st.exc[u] > 0 && st.lab[u] < g.dinf && region_touched<CONN>(g, st, r)) st.active[r] = 1;
-        }
-    } else {
-        for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < (long long)g.n; v += stride) {
-            const int x = (int)(v % g.X), y = (int)(v / g.X);
-            int l = st.lab[v];
-            if (l > gap && l < g.dinf) {
-                l = g.dinf;
-                st.lab[v] = l;
-            }
-            const int lx = x & (g.tx - 1), ly = y & (g.ty - 1);
-            if (lx != 0 && lx != g.tx - 1 && ly != 0 && ly != g.ty - 1) continue;
-            const int r = (y >> g.sy) * g.RX + (x >> g.sx);
-            if (l < g.dinf && st.exc[v] > 0 && region_touched<CONN>(g, st, r)) st.active[r] = 1;
-        }
-    }
-}
 
 // count the active regions for the host, reset the per-sweep flags
 __global__ void finish_flags_kernel(const DevState st, int nreg) {
@@ -711,7 +687,7 @@ __global__ void post_batch_kernel(const Inst *insts, const int2 *regs, int nregs
     for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < nregs; i += nw) {
         const int2 w = regs[i];
         if (done[w.x] || insts[w.x].conn != CONN) continue;
-        post_region_warp<CONN>(insts[w.x].g, insts[w.x].st, w.y, insts[w.x].st.ctr[kGap]);
+        post_region_warp<CONN, false>(insts[w.x].g, insts[w.x].st, w.y, insts[w.x].st.ctr[kGap]);
     }
 }
 
@@ -742,14 +718,6 @@ __global__ void batch_relabel_end_kernel(const Inst *insts, unsigned char *done,
         if (done[i]) continue;
         if (insts[i].st.ctr[kActiveRegions] == 0) done[i] = 1;
         else atomicAdd(any, 1);
-    }
-}
-
-// per-sweep flags are cleared after post has read them
-__global__ void clear_flags_kernel(const DevState st, int nreg) {
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nreg; r += gridDim.x * blockDim.x) {
-        st.disc[r] = 0;
-        st.left_active[r] = 0;
     }
 }
 
@@ -849,20 +817,12 @@ static cudaError_t launch_validate(mf_grid *h, int *flags) {
 }
 template <int CONN>
 static cudaError_t launch_fuse_post(mf_grid *h, bool gap_on, cudaStream_t st) {
-    if (CONN != 6 && !is_paper(CONN)) {
-        const long long items = (long long)h->g.nreg * (2 * h->g.tx + 2 * (h->g.ty - 2));
-        const int fb = (int)std::min<long long>((items + 255) / 256, device_sms() * 8);
-        fuse2d_kernel<CONN><<<fb, 256, 0, st>>>(h->g, h->st);
-        if (gap_on) gap_find_kernel<<<1, 1024, 0, st>>>(h->st);
-        post2d_kernel<CONN><<<device_sms() * 8, 256, 0, st>>>(h->g, h->st);
-        finish_flags_kernel<<<(h->g.nreg + 255) / 256, 256, 0, st>>>(h->st, h->g.nreg);
-        return cudaGetLastError();
-    }
-    const int wb = (int)std::min<long long>(((long long)h->g.nreg + 7) / 8, (long long)device_sms() * 8);
-    fuse_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st);
+    const int split = surface_split(h->g, CONN);
+    const int wb = (int)std::min<long long>(((long long)h->g.nreg * split + 7) / 8, (long long)device_sms() * 8);
+    fuse_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st, split);
     if (gap_on) gap_find_kernel<<<1, 1024, 0, st>>>(h->st);
-    post_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st);
-    clear_flags_kernel<<<(h->g.nreg + 255) / 256, 256, 0, st>>>(h->st, h->g.nreg);
+    post_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st, split);
+    finish_flags_kernel<<<(h->g.nreg + 255) / 256, 256, 0, st>>>(h->st, h->g.nreg);
     return cudaGetLastError();
 }
 template <int CONN>
