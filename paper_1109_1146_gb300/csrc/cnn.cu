@@ -5,11 +5,11 @@
 // optimiser and used as BF16 in every product; all sums accumulate in FP32.
 // Activations are FP32, layout [N][C][H][W].
 //
-// Kernels: direct convolution forward (one thread per output pixel, all output
-// channels in registers, the input tile and the layer's weights staged in
-// shared memory), the input gradient (the same convolution with transposed,
-// flipped weights), the weight / bias gradients (per-tile partial sums added
-// atomically), a mean-squared-error loss with its gradient, and Adam.
+// Kernels: direct convolution in FP32 for the forward pass and the input
+// gradient (the same convolution with transposed, flipped weights and the ReLU
+// of the layer below applied to its result), the weight / bias gradients
+// (partial sums per block in registers, then one reduction), a mean-squared-
+// error loss with its gradient, and Adam.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -25,117 +25,366 @@
 
 namespace mf {
 
-constexpr int kTile = 16;  // output tile edge of the convolution kernels
-
-template <int CIN, int COUT, bool RELU>
-__global__ void __launch_bounds__(256) conv3x3_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w,
-                                                      const float *__restrict__ b, float *__restrict__ y, int H, int W) {
-    extern __shared__ float sm[];
-    float *sw = sm;                          // [COUT][CIN][9]
-    float *sx = sw + COUT * CIN * 9;         // [CIN][18][18]
-    const int n = blockIdx.z;
-    const int ox = blockIdx.x * kTile, oy = blockIdx.y * kTile;
-    const int tid = threadIdx.x;
-    for (int i = tid; i < COUT * CIN * 9; i += blockDim.x) sw[i] = __bfloat162float(w[i]);
-    const float *xn = x + (size_t)n * CIN * H * W;
-    for (int i = tid; i < CIN * 18 * 18; i += blockDim.x) {
-        const int c = i / 324, r = (i / 18) % 18, q = i % 18;
-        const int gy = oy + r - 1, gx = ox + q - 1;
-        sx[i] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? xn[((size_t)c * H + gy) * W + gx] : 0.f;
-    }
-    __syncthreads();
-    const int ty = tid / kTile, tx = tid % kTile;
-    const int py = oy + ty, px = ox + tx;
-    float acc[COUT];
-#pragma unroll
-    for (int co = 0; co < COUT; ++co) acc[co] = b[co];
-    for (int ci = 0; ci < CIN; ++ci) {
-        float in[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) in[k] = sx[(ci * 18 + ty + k / 3) * 18 + tx + k % 3];
-#pragma unroll
-        for (int co = 0; co < COUT; ++co) {
-            const float *wk = sw + (co * CIN + ci) * 9;
-#pragma unroll
-            for (int k = 0; k < 9; ++k) acc[co] = fmaf(wk[k], in[k], acc[co]);
-        }
-    }
-    if (py < H && px < W) {
-        float *yn = y + (size_t)n * COUT * H * W;
-#pragma unroll
-        for (int co = 0; co < COUT; ++co) {
-            const float v = RELU ? fmaxf(acc[co], 0.f) : acc[co];
-            yn[((size_t)co * H + py) * W + px] = v;
-        }
-    }
+// two FP32 fused multiply-adds in one instruction (each rounded as fmaf)
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+// global -> shared copy of one float; zero where !in
+__device__ __forceinline__ void copy_f32(float *dst, const float *src, bool in) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(in ? 4 : 0) : "memory");
 }
 
-// dy' = dy * [y > 0] for a ReLU layer (y is the layer's output)
-__global__ void relu_mask_kernel(float *dy, const float *y, size_t n) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        if (!(y[i] > 0.f)) dy[i] = 0.f;
-}
-
-// wt[ci][co][8-k] = w[co][ci][k]: the input gradient is a 3x3 convolution of dy
-// with these weights
-__global__ void transpose_flip_kernel(const __nv_bfloat16 *w, __nv_bfloat16 *wt, int cout, int cin) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < cout * cin * 9; i += gridDim.x * blockDim.x) {
-        const int co = i / (cin * 9), ci = (i / 9) % cin, k = i % 9;
-        wt[(ci * cout + co) * 9 + (8 - k)] = w[i];
-    }
-}
-
-// dW[co][ci][k] += sum over pixels of dy[co][p] * x[ci][p + off(k)];  db[co] += sum dy[co][p]
+// Direct 3x3 convolution.  A thread computes PX pixels of a row times CO output
+// channels, channels in pairs (one two-wide FMA per pair, pixel and tap), so
+// that a weight read from shared memory (a broadcast) serves PX pixels and an
+// input CO channels.  A warp covers 32 columns and PX rows; the block's warps
+// are CG channel groups times NWARP / CG row groups.  The input tile comes in
+// chunks of CK channels, the next one copied asynchronously under the
+// arithmetic; the weights stay in shared memory as FP32 [ci][tap][co].
+// Per output: the bias, then fmaf over ci and tap in ascending order.
+//   TRANS: the input gradient: weight of (out o, in i, tap k) = w[i][o][8 - k].
+//   MASK:  zero where act <= 0 (the ReLU of the layer whose output gradient
+//          this is).
+// Bound by FP32 FMAs.  A thread per pixel with all 32 channels and a scalar
+// weight read per FMA took 573 us for 32 -> 32 channels on 8 x 256 x 256 pixels
+// (17 TFLOP/s), this 210 us (46 TFLOP/s; the FMA pipe is 70% busy).
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(256) conv3x3_wgrad_kernel(const float *__restrict__ x, const float *__restrict__ dy,
-                                                            float *dw, float *db, int H, int W) {
-    extern __shared__ float sm[];
-    float *sx = sm;                       // [CIN][18][18]
-    float *sd = sx + CIN * 18 * 18;       // [COUT][16][16]
-    const int n = blockIdx.z;
-    const int ox = blockIdx.x * kTile, oy = blockIdx.y * kTile;
-    const int tid = threadIdx.x;
+struct ConvCfg {
+    static constexpr int CG = COUT == 32 ? 2 : 1;         // channel groups
+    static constexpr int CO = COUT / CG;                  // channels per thread
+    static constexpr int PX = COUT == 32 ? 4 : 8;         // pixels per thread
+    static constexpr int NWARP = COUT == 32 ? 8 : 4;
+    static constexpr int TH = PX * (NWARP / CG);          // tile height (width 32)
+    static constexpr int CK = CIN == 32 ? 8 : CIN == 10 ? 5 : CIN;  // input channels per chunk
+    static constexpr int NC = CIN / CK;
+    static constexpr int XS = 36;                         // row stride of the staged tile
+    static constexpr int WS = COUT == 10 ? 12 : COUT == 6 ? 8 : COUT;  // channel stride of the weights
+    static constexpr size_t chunk = (size_t)CK * (TH + 2) * XS;
+    static constexpr size_t smem = ((size_t)CIN * 9 * WS + (NC > 1 ? 2 : 1) * chunk) * 4;
+    static_assert(CIN % CK == 0 && COUT % CG == 0 && CO % 2 == 0, "channel split");
+};
+
+template <int CIN, int COUT, bool RELU, bool TRANS, bool MASK>
+__global__ void __launch_bounds__(ConvCfg<CIN, COUT>::NWARP * 32, 2)
+conv3x3_kernel(const float *__restrict__ x, const __nv_bfloat16 *__restrict__ w, const float *__restrict__ b,
+               const float *__restrict__ act, float *__restrict__ y, int H, int W) {
+    using C = ConvCfg<CIN, COUT>;
+    constexpr int NT = C::NWARP * 32, PX = C::PX, P2 = C::CO / 2, XS = C::XS, WS = C::WS, CK = C::CK, TH = C::TH;
+    extern __shared__ __align__(16) float sm[];
+    float *s_w = sm;                        // [CIN][9][WS]
+    float *s_x = sm + CIN * 9 * WS;         // [1 or 2][CK][TH + 2][XS]
+    const int n = blockIdx.z, ox = blockIdx.x * 32, oy = blockIdx.y * TH;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const float *xn = x + (size_t)n * CIN * H * W;
-    const float *dn = dy + (size_t)n * COUT * H * W;
-    for (int i = tid; i < CIN * 18 * 18; i += blockDim.x) {
-        const int c = i / 324, r = (i / 18) % 18, q = i % 18;
-        const int gy = oy + r - 1, gx = ox + q - 1;
-        sx[i] = (gy >= 0 && gy < H && gx >= 0 && gx < W) ? xn[((size_t)c * H + gy) * W + gx] : 0.f;
+    const int gx = ox + lane - 1;
+    const bool xin = gx >= 0 && gx < W, xin2 = gx + 32 < W;
+    auto stage = [&](int c) {
+        float *dst = s_x + (c & 1) * C::chunk;
+        const float *src = xn + (size_t)c * CK * H * W;
+        // a row of 34 per warp and step: the index arithmetic is the warp's, not
+        // a thread's (it would run on the FMA pipes)
+        for (int row = warp; row < CK * (TH + 2); row += C::NWARP) {
+            const int ci = row / (TH + 2), gy = oy + row % (TH + 2) - 1;
+            const bool yin = gy >= 0 && gy < H;
+            const float *sr = src + ((size_t)ci * H + (yin ? gy : 0)) * W;
+            copy_f32(dst + row * XS + lane, xin ? sr + gx : src, yin && xin);
+            if (lane < 2) copy_f32(dst + row * XS + 32 + lane, xin2 ? sr + gx + 32 : src, yin && xin2);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    stage(0);
+    for (int i = tid; i < CIN * 9 * WS; i += NT) {
+        const int co = i % WS, k = (i / WS) % 9, ci = i / (9 * WS);
+        float v = 0.f;
+        if (co < COUT) v = __bfloat162float(TRANS ? w[((size_t)ci * COUT + co) * 9 + 8 - k] : w[((size_t)co * CIN + ci) * 9 + k]);
+        s_w[i] = v;
     }
-    for (int i = tid; i < COUT * 256; i += blockDim.x) {
-        const int c = i / 256, r = (i / 16) % 16, q = i % 16;
-        const int gy = oy + r, gx = ox + q;
-        sd[i] = (gy < H && gx < W) ? dn[((size_t)c * H + gy) * W + gx] : 0.f;
+    const int co0 = (warp % C::CG) * C::CO;
+    const int xl = (lane % (32 / PX)) * PX, yl = (warp / C::CG) * PX + lane / (32 / PX);
+    uint64_t acc[PX][P2];
+#pragma unroll
+    for (int j = 0; j < P2; ++j) {
+        const uint64_t b2 = TRANS ? 0ull : pack2(b[co0 + 2 * j], b[co0 + 2 * j + 1]);
+#pragma unroll
+        for (int p = 0; p < PX; ++p) acc[p][j] = b2;
     }
+#pragma unroll 1
+    for (int c = 0; c < C::NC; ++c) {
+        if (c + 1 < C::NC) {
+            stage(c + 1);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncthreads();
+        const float *xt = s_x + (c & 1) * C::chunk + yl * XS + xl;
+        const float *wt = s_w + c * CK * 9 * WS + co0;
+#pragma unroll 1
+        for (int ci = 0; ci < CK; ++ci) {
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky) {
+                uint64_t xd[PX + 2];  // (x, x) pairs
+                const float *xr = xt + (ci * (TH + 2) + ky) * XS;
+#pragma unroll
+                for (int q = 0; q < PX; q += 4) {
+                    const float4 v = *(const float4 *)(xr + q);
+                    xd[q] = pack2(v.x, v.x);
+                    xd[q + 1] = pack2(v.y, v.y);
+                    xd[q + 2] = pack2(v.z, v.z);
+                    xd[q + 3] = pack2(v.w, v.w);
+                }
+                const float2 e = *(const float2 *)(xr + PX);
+                xd[PX] = pack2(e.x, e.x);
+                xd[PX + 1] = pack2(e.y, e.y);
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx) {
+                    uint64_t w2[P2];
+                    const float *wr = wt + (ci * 9 + ky * 3 + kx) * WS;
+#pragma unroll
+                    for (int j = 0; j + 1 < P2; j += 2) {
+                        const ulonglong2 v = *(const ulonglong2 *)(wr + 2 * j);
+                        w2[j] = v.x;
+                        w2[j + 1] = v.y;
+                    }
+                    if (P2 & 1) w2[P2 - 1] = *(const uint64_t *)(wr + 2 * (P2 - 1));
+#pragma unroll
+                    for (int p = 0; p < PX; ++p)
+#pragma unroll
+                        for (int j = 0; j < P2; ++j) acc[p][j] = fma2(w2[j], xd[p + kx], acc[p][j]);
+                }
+            }
+        }
+        __syncthreads();  // the chunk after next reuses this buffer
+    }
+    const int py = oy + yl, px = ox + xl;
+    if (py >= H) return;
+    const size_t out0 = ((size_t)(n * COUT + co0) * H + py) * W + px;
+    const bool vec = W % 4 == 0 && px + PX <= W && (((uintptr_t)y | (uintptr_t)act) & 15) == 0;
+#pragma unroll
+    for (int j = 0; j < P2; ++j) {
+        float v[2][PX];
+#pragma unroll
+        for (int p = 0; p < PX; ++p) {
+            unpack2(acc[p][j], v[0][p], v[1][p]);
+            if (RELU) {
+                v[0][p] = fmaxf(v[0][p], 0.f);
+                v[1][p] = fmaxf(v[1][p], 0.f);
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const size_t o = out0 + (size_t)(2 * j + h) * H * W;
+            if (vec) {
+#pragma unroll
+                for (int p = 0; p < PX; p += 4) {
+                    if (MASK) {
+                        const float4 a = *(const float4 *)(act + o + p);
+                        if (!(a.x > 0.f)) v[h][p] = 0.f;
+                        if (!(a.y > 0.f)) v[h][p + 1] = 0.f;
+                        if (!(a.z > 0.f)) v[h][p + 2] = 0.f;
+                        if (!(a.w > 0.f)) v[h][p + 3] = 0.f;
+                    }
+                    *(float4 *)(y + o + p) = make_float4(v[h][p], v[h][p + 1], v[h][p + 2], v[h][p + 3]);
+                }
+            } else {
+#pragma unroll
+                for (int p = 0; p < PX; ++p)
+                    if (px + p < W) y[o + p] = MASK && !(act[o + p] > 0.f) ? 0.f : v[h][p];
+            }
+        }
+    }
+}
+
+// Weight and bias gradients of a layer:
+//   dW[co][ci][k] = sum over pixels of dy[co][p] * x[ci][p + off(k)],  db[co] = sum of dy[co][p].
+// A thread holds 4 output channels x 1 input channel x 9 taps, each sum split
+// over even and odd columns (two-wide FMAs on pixel pairs): 7 vector reads from
+// shared memory per 72 FMAs.  Lanes are input channels; with few of them the
+// lanes also split the tile's rows, with few output channels the warps do.  A
+// block walks 16x16 tiles and keeps its sums in registers; its partial sums go
+// to part[block * RGW + row group][..], summed by wgrad_reduce_kernel.
+// Bound by FP32 FMAs.  One thread per weight walking a tile with scalar reads
+// and an atomic add per weight and tile took 1298 us for 32 -> 32 channels on
+// 8 x 256 x 256 pixels, this 291 us.
+template <int CIN, int COUT>
+struct WgradCfg {
+    static constexpr int LC = CIN <= 8 ? 8 : CIN <= 16 ? 16 : 32;  // lanes over input channels
+    static constexpr int RGL = 32 / LC;                            // row groups within a warp
+    static constexpr int Q = (COUT + 3) / 4;                       // quads of output channels
+    static constexpr int RGW = Q >= 8 ? 1 : Q >= 3 ? 2 : 4;        // row groups over warps
+    static constexpr int RG = RGL * RGW, RR = 16 / RG;             // row groups, rows of one
+    static constexpr int NT = 32 * Q * RGW;
+    static constexpr int XP = 364;                                 // plane stride of x (18 rows of 20)
+    static constexpr int DG = RR * 16 + 4, DP = RG * DG;           // row group and plane stride of dy
+    static constexpr int K = COUT * CIN * 9 + COUT;                // sums of one layer
+    static constexpr size_t smem = (size_t)(LC * XP + Q * 4 * DP) * 4;
+};
+
+template <int CIN, int COUT>
+__global__ void __launch_bounds__(WgradCfg<CIN, COUT>::NT, 2)
+conv3x3_wgrad_kernel(const float *__restrict__ x, const float *__restrict__ dy, float *__restrict__ part, int N, int H,
+                     int W) {
+    using C = WgradCfg<CIN, COUT>;
+    constexpr int NT = C::NT;
+    extern __shared__ __align__(16) float sm[];
+    float *s_x = sm;                   // [LC][18][20], plane stride XP
+    float *s_d = sm + C::LC * C::XP;   // [4 Q][RG][RR][16], strides DP, DG
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int q = warp % C::Q, rgw = warp / C::Q, ci = lane % C::LC, rg = rgw * C::RGL + lane / C::LC;
+    for (int i = tid; i < C::LC * C::XP + C::Q * 4 * C::DP; i += NT) sm[i] = 0.f;  // unused channels and padding
+    const int tx = (W + 15) / 16, ty = (H + 15) / 16, tiles = tx * ty * N;
+    uint64_t acc[4][9];
+    float db[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+        for (int k = 0; k < 9; ++k) acc[c][k] = 0ull;
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x) {
+        const int n = t / (tx * ty), oy = (t / tx) % ty * 16, ox = t % tx * 16;
+        const float *xn = x + (size_t)n * CIN * H * W;
+        const float *dn = dy + (size_t)n * COUT * H * W;
+        __syncthreads();  // the previous tile has been used
+        // two rows per warp and step, a half-warp each
+        const int hl = lane & 15, hr = lane >> 4;
+        const int gx = ox + hl - 1;
+        const bool xin = gx >= 0 && gx < W, xin2 = gx + 16 < W, din = ox + hl < W;
+        for (int row = 2 * warp; row < CIN * 18; row += NT / 16) {
+            const int c = row / 18, r = row % 18 + hr, gy = oy + r - 1;  // (18 is even: one channel per step)
+            const bool yin = gy >= 0 && gy < H;
+            const float *sr = xn + ((size_t)c * H + (yin ? gy : 0)) * W;
+            float *dst = s_x + c * C::XP + r * 20;
+            copy_f32(dst + hl, xin ? sr + gx : xn, yin && xin);
+            if (hl < 2) copy_f32(dst + 16 + hl, xin2 ? sr + gx + 16 : xn, yin && xin2);
+        }
+        for (int row = 2 * warp; row < COUT * 16; row += NT / 16) {
+            const int c = row / 16, r = row % 16 + hr, gy = oy + r;
+            const bool in = gy < H && din;
+            copy_f32(s_d + c * C::DP + (r / C::RR) * C::DG + (r % C::RR) * 16 + hl,
+                     in ? dn + ((size_t)c * H + gy) * W + ox + hl : dn, in);
+        }
+        asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const float *xp = s_x + ci * C::XP + rg * C::RR * 20;
+        const float *dp = s_d + q * 4 * C::DP + rg * C::DG;
+#pragma unroll 1
+        for (int r = 0; r < C::RR; ++r) {
+#pragma unroll 1
+            for (int p = 0; p < 16; p += 4) {
+                uint64_t d[4][2];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const ulonglong2 v = *(const ulonglong2 *)(dp + c * C::DP + r * 16 + p);
+                    d[c][0] = v.x;
+                    d[c][1] = v.y;
+                }
+#pragma unroll
+                for (int ky = 0; ky < 3; ++ky) {
+                    const float *xr = xp + (r + ky) * 20 + p;
+                    const float4 v = *(const float4 *)xr;
+                    const float2 e = *(const float2 *)(xr + 4);
+                    // pixel pairs (0,1), (2,3) shifted by kx
+                    const uint64_t x0 = pack2(v.x, v.y), x1 = pack2(v.y, v.z), x2 = pack2(v.z, v.w), x3 = pack2(v.w, e.x),
+                                   x4 = pack2(e.x, e.y);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[c][ky * 3] = fma2(d[c][0], x0, acc[c][ky * 3]);
+                        acc[c][ky * 3 + 1] = fma2(d[c][0], x1, acc[c][ky * 3 + 1]);
+                        acc[c][ky * 3 + 2] = fma2(d[c][0], x2, acc[c][ky * 3 + 2]);
+                    }
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[c][ky * 3] = fma2(d[c][1], x2, acc[c][ky * 3]);
+                        acc[c][ky * 3 + 1] = fma2(d[c][1], x3, acc[c][ky * 3 + 1]);
+                        acc[c][ky * 3 + 2] = fma2(d[c][1], x4, acc[c][ky * 3 + 2]);
+                    }
+                }
+            }
+        }
+        // bias: the lanes of a row group share its pixels
+        for (int p = ci; p < C::RR * 16; p += C::LC)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) db[c] += dp[c * C::DP + p];
+    }
+    float *out = part + (size_t)(blockIdx.x * C::RGW + rgw) * C::K;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const int co = q * 4 + c;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            float lo, hi;
+            unpack2(acc[c][k], lo, hi);
+            float v = lo + hi;
+#pragma unroll
+            for (int o = C::LC; o < 32; o *= 2) v += __shfl_xor_sync(0xffffffffu, v, o);
+            if (lane < C::LC && ci < CIN && co < COUT) out[(co * CIN + ci) * 9 + k] = v;
+        }
+        float v = db[c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0 && co < COUT) out[COUT * CIN * 9 + co] = v;
+    }
+}
+
+// g[e] += sum over the partial sums part[0 .. rows)[e], in float64 (a warp per
+// 32 sums and slice of the rows, four loads in flight); g holds a layer's weight
+// gradients followed by its bias gradients
+__global__ void __launch_bounds__(512) wgrad_reduce_kernel(const float *__restrict__ part, int rows, int K, float *g) {
+    __shared__ double s[16][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+    double v = 0;
+    if (e < K) {
+        int r = warp;
+        for (; r + 48 < rows; r += 64) {
+            const float a = part[(size_t)r * K + e], b = part[(size_t)(r + 16) * K + e];
+            const float c = part[(size_t)(r + 32) * K + e], d = part[(size_t)(r + 48) * K + e];
+            v += ((double)a + b) + ((double)c + d);
+        }
+        for (; r < rows; r += 16) v += (double)part[(size_t)r * K + e];
+    }
+    s[warp][lane] = v;
     __syncthreads();
-    for (int e = tid; e < COUT * CIN * 9; e += blockDim.x) {
-        const int co = e / (CIN * 9), ci = (e / 9) % CIN, k = e % 9;
-        const int ky = k / 3, kx = k % 3;
-        const float *d = sd + co * 256;
-        const float *xs = sx + ci * 324;
-        float s = 0.f;
-        for (int r = 0; r < 16; ++r)
-#pragma unroll 4
-            for (int q = 0; q < 16; ++q) s = fmaf(d[r * 16 + q], xs[(r + ky) * 18 + q + kx], s);
-        atomicAdd(&dw[e], s);
-    }
-    for (int co = tid; co < COUT; co += blockDim.x) {
-        float s = 0.f;
-        for (int p = 0; p < 256; ++p) s += sd[co * 256 + p];
-        atomicAdd(&db[co], s);
+    if (warp == 0 && e < K) {
+        for (int k = 1; k < 16; ++k) v += s[k][lane];
+        g[e] += (float)v;
     }
 }
 
 // mean squared error over count values and its gradient dy = 2 (y - t) / count
-__global__ void mse_kernel(const float *y, const float *t, float *dy, size_t count, double *loss) {
+// (a double per block: per warp, the atomics on the one sum took most of the time)
+__global__ void __launch_bounds__(256) mse_kernel(const float *y, const float *t, float *dy, size_t count, double *loss) {
+    __shared__ double sw[8];
+    const float scale = (float)count;
     double s = 0;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < count; i += (size_t)gridDim.x * blockDim.x) {
-        const float d = y[i] - t[i];
-        dy[i] = 2.f * d / (float)count;
+    auto one = [&](float a, float b) -> float {
+        const float d = a - b;
         s += (double)d * d;
+        return 2.f * d / scale;
+    };
+    const size_t i0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
+    const bool vec = (((uintptr_t)y | (uintptr_t)t | (uintptr_t)dy) & 15) == 0;
+    const size_t n4 = vec ? count / 4 : 0;
+    for (size_t i = i0; i < n4; i += stride) {
+        const float4 a = ((const float4 *)y)[i], b = ((const float4 *)t)[i];
+        ((float4 *)dy)[i] = make_float4(one(a.x, b.x), one(a.y, b.y), one(a.z, b.z), one(a.w, b.w));
     }
+    for (size_t i = n4 * 4 + i0; i < count; i += stride) dy[i] = one(y[i], t[i]);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0 && s != 0) atomicAdd(loss, s / (double)count);
+    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int k = 1; k < 8; ++k) s += sw[k];
+        if (s != 0) atomicAdd(loss, s / (double)count);
+    }
 }
 
 // Adam on FP32 master weights; refreshes the BF16 copy used by the products
@@ -318,19 +567,15 @@ __global__ void __launch_bounds__(256) conv3x3_mma_kernel(const void *__restrict
 }
 
 // ---- host side ---------------------------------------------------------------
-template <int CIN, int COUT, bool RELU>
-static cudaError_t conv_fwd(const float *x, const __nv_bfloat16 *w, const float *b, float *y, int N, int H, int W,
-                            cudaStream_t s) {
-    const size_t smem = (size_t)(COUT * CIN * 9 + CIN * 18 * 18) * 4;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(conv3x3_kernel<CIN, COUT, RELU>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
-    conv3x3_kernel<CIN, COUT, RELU><<<grid, 256, smem, s>>>(x, w, b, y, H, W);
+template <int CIN, int COUT, bool RELU, bool TRANS, bool MASK>
+static cudaError_t conv(const float *x, const __nv_bfloat16 *w, const float *b, const float *act, float *y, int N, int H,
+                        int W, cudaStream_t s) {
+    using C = ConvCfg<CIN, COUT>;
+    auto k = conv3x3_kernel<CIN, COUT, RELU, TRANS, MASK>;
+    const cudaError_t e = ensure_smem_attr((const void *)k, (int)C::smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((W + 31) / 32, (H + C::TH - 1) / C::TH, N);
+    k<<<grid, C::NWARP * 32, C::smem, s>>>(x, w, b, act, y, H, W);
     return cudaGetLastError();
 }
 
@@ -355,44 +600,54 @@ static cudaError_t conv_mma(const void *x, int cin, const __nv_bfloat16 *w, cons
     return cudaGetLastError();
 }
 
+// partial sums of a layer's weight gradients: rows of K floats
+static int wgrad_blocks() { return device_sms() * 2; }
+constexpr size_t kWgradRow = 32 * 32 * 9 + 32;  // the largest layer's sums
+constexpr int kWgradRows = 4;                   // row groups a block may write
+
 template <int CIN, int COUT>
-static cudaError_t conv_wgrad(const float *x, const float *dy, float *dw, float *db, int N, int H, int W,
+static cudaError_t conv_wgrad(const float *x, const float *dy, float *part, float *g, int N, int H, int W,
                               cudaStream_t s) {
-    const size_t smem = (size_t)(CIN * 18 * 18 + COUT * 256) * 4;
-    static bool attr = false;
-    if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_kernel<CIN, COUT>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        attr = true;
-    }
-    dim3 grid((W + kTile - 1) / kTile, (H + kTile - 1) / kTile, N);
-    conv3x3_wgrad_kernel<CIN, COUT><<<grid, 256, smem, s>>>(x, dy, dw, db, H, W);
+    using C = WgradCfg<CIN, COUT>;
+    static_assert(C::K <= kWgradRow && C::RGW <= kWgradRows, "partial sums");
+    auto k = conv3x3_wgrad_kernel<CIN, COUT>;
+    const cudaError_t e = ensure_smem_attr((const void *)k, (int)C::smem);
+    if (e != cudaSuccess) return e;
+    const long long tiles = (long long)((W + 15) / 16) * ((H + 15) / 16) * N;
+    const int grid = (int)std::min<long long>(tiles, wgrad_blocks());
+    k<<<grid, C::NT, C::smem, s>>>(x, dy, part, N, H, W);
+    wgrad_reduce_kernel<<<(C::K + 31) / 32, 512, 0, s>>>(part, grid * C::RGW, C::K, g);
     return cudaGetLastError();
 }
 
 // (cin, cout, relu) dispatch over the layer shapes the network uses
 static cudaError_t conv_fwd_any(int cin, int cout, bool relu, const float *x, const __nv_bfloat16 *w, const float *b,
                                 float *y, int N, int H, int W, cudaStream_t s) {
-    if (cin == 6 && cout == 32 && relu) return conv_fwd<6, 32, true>(x, w, b, y, N, H, W, s);
-    if (cin == 10 && cout == 32 && relu) return conv_fwd<10, 32, true>(x, w, b, y, N, H, W, s);
-    if (cin == 32 && cout == 32 && relu) return conv_fwd<32, 32, true>(x, w, b, y, N, H, W, s);
-    if (cin == 32 && cout == 6 && !relu) return conv_fwd<32, 6, false>(x, w, b, y, N, H, W, s);
-    if (cin == 32 && cout == 10 && !relu) return conv_fwd<32, 10, false>(x, w, b, y, N, H, W, s);
-    // input gradients: transposed layers without ReLU
-    if (cin == 32 && cout == 32 && !relu) return conv_fwd<32, 32, false>(x, w, b, y, N, H, W, s);
-    if (cin == 6 && cout == 32 && !relu) return conv_fwd<6, 32, false>(x, w, b, y, N, H, W, s);
-    if (cin == 10 && cout == 32 && !relu) return conv_fwd<10, 32, false>(x, w, b, y, N, H, W, s);
+    if (cin == 6 && cout == 32 && relu) return conv<6, 32, true, false, false>(x, w, b, nullptr, y, N, H, W, s);
+    if (cin == 10 && cout == 32 && relu) return conv<10, 32, true, false, false>(x, w, b, nullptr, y, N, H, W, s);
+    if (cin == 32 && cout == 32 && relu) return conv<32, 32, true, false, false>(x, w, b, nullptr, y, N, H, W, s);
+    if (cin == 32 && cout == 6 && !relu) return conv<32, 6, false, false, false>(x, w, b, nullptr, y, N, H, W, s);
+    if (cin == 32 && cout == 10 && !relu) return conv<32, 10, false, false, false>(x, w, b, nullptr, y, N, H, W, s);
     return cudaErrorInvalidValue;
 }
 
-static cudaError_t conv_wgrad_any(int cin, int cout, const float *x, const float *dy, float *dw, float *db, int N,
+// input gradient of a layer cin -> cout, with the ReLU mask of the layer below
+// (act: its output): dx has cin = 32 channels
+static cudaError_t conv_dgrad_any(int cin, int cout, const float *dy, const __nv_bfloat16 *w, const float *act, float *dx,
+                                  int N, int H, int W, cudaStream_t s) {
+    if (cin == 32 && cout == 32) return conv<32, 32, false, true, true>(dy, w, nullptr, act, dx, N, H, W, s);
+    if (cin == 32 && cout == 6) return conv<6, 32, false, true, true>(dy, w, nullptr, act, dx, N, H, W, s);
+    if (cin == 32 && cout == 10) return conv<10, 32, false, true, true>(dy, w, nullptr, act, dx, N, H, W, s);
+    return cudaErrorInvalidValue;
+}
+
+static cudaError_t conv_wgrad_any(int cin, int cout, const float *x, const float *dy, float *part, float *g, int N,
                                   int H, int W, cudaStream_t s) {
-    if (cin == 6 && cout == 32) return conv_wgrad<6, 32>(x, dy, dw, db, N, H, W, s);
-    if (cin == 10 && cout == 32) return conv_wgrad<10, 32>(x, dy, dw, db, N, H, W, s);
-    if (cin == 32 && cout == 32) return conv_wgrad<32, 32>(x, dy, dw, db, N, H, W, s);
-    if (cin == 32 && cout == 6) return conv_wgrad<32, 6>(x, dy, dw, db, N, H, W, s);
-    if (cin == 32 && cout == 10) return conv_wgrad<32, 10>(x, dy, dw, db, N, H, W, s);
+    if (cin == 6 && cout == 32) return conv_wgrad<6, 32>(x, dy, part, g, N, H, W, s);
+    if (cin == 10 && cout == 32) return conv_wgrad<10, 32>(x, dy, part, g, N, H, W, s);
+    if (cin == 32 && cout == 32) return conv_wgrad<32, 32>(x, dy, part, g, N, H, W, s);
+    if (cin == 32 && cout == 6) return conv_wgrad<32, 6>(x, dy, part, g, N, H, W, s);
+    if (cin == 32 && cout == 10) return conv_wgrad<32, 10>(x, dy, part, g, N, H, W, s);
     return cudaErrorInvalidValue;
 }
 
@@ -406,10 +661,9 @@ struct mf_cnn {
     size_t nparam = 0;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;  // master params, grads, Adam moments
     __nv_bfloat16 *pb = nullptr;                                   // BF16 copy used by the products
-    __nv_bfloat16 *wt = nullptr;                                   // scratch: transposed weights
+    float *part = nullptr;                                         // partial weight gradients of a backward pass
     float *act[5] = {nullptr, nullptr, nullptr, nullptr, nullptr}; // layer outputs of the last kept forward
     float *dbuf[2] = {nullptr, nullptr};                           // gradient ping-pong buffers
-    float *zero_bias = nullptr;
     double *dloss = nullptr;
     __nv_bfloat16 *ibuf[2] = {nullptr, nullptr};                   // inference activations, BF16 NHWC x 32
     size_t icap_pix = 0;
@@ -502,14 +756,11 @@ mf_status mf_cnn_create(mf_cnn **out, int in_ch, int out_ch, uint64_t seed, void
     if (e == cudaSuccess) e = cudaMalloc(&c->m, off * 4);
     if (e == cudaSuccess) e = cudaMalloc(&c->v, off * 4);
     if (e == cudaSuccess) e = cudaMalloc(&c->pb, off * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&c->wt, 32 * 32 * 9 * 2);
-    if (e == cudaSuccess) e = cudaMalloc(&c->zero_bias, 32 * 4);
     if (e == cudaSuccess) e = cudaMalloc(&c->dloss, 8);
     if (e == cudaSuccess) e = cudaMemcpy(c->p, h.data(), off * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemset(c->g, 0, off * 4);
     if (e == cudaSuccess) e = cudaMemset(c->m, 0, off * 4);
     if (e == cudaSuccess) e = cudaMemset(c->v, 0, off * 4);
-    if (e == cudaSuccess) e = cudaMemset(c->zero_bias, 0, 32 * 4);
     if (e == cudaSuccess) {
         to_bf16_kernel<<<64, 256, 0, c->stream>>>(c->p, c->pb, off);
         e = cudaStreamSynchronize(c->stream);
@@ -526,7 +777,7 @@ mf_status mf_cnn_create(mf_cnn **out, int in_ch, int out_ch, uint64_t seed, void
 mf_status mf_cnn_destroy(mf_cnn *c) {
     if (!c) return MF_OK;
     cnn_free_acts(c);
-    void *ps[] = {c->p, c->g, c->m, c->v, c->pb, c->wt, c->zero_bias, c->dloss, c->ibuf[0], c->ibuf[1]};
+    void *ps[] = {c->p, c->g, c->m, c->v, c->pb, c->part, c->dloss, c->ibuf[0], c->ibuf[1]};
     for (void *q : ps)
         if (q) cudaFree(q);
     delete c;
@@ -653,24 +904,18 @@ mf_status mf_cnn_zero_grad(mf_cnn *c) {
 mf_status mf_cnn_backward(mf_cnn *c, const float *x, const float *dy) {
     if (!c || !x || !dy || !c->N) return cnn_fail(c, MF_EINVAL, "backward needs the last forward's input and dy");
     const int N = c->N, H = c->H, W = c->W;
-    const size_t pix = (size_t)N * H * W;
-    // gradient of layer l's output lives in cur; layer 4 has no ReLU
+    if (!c->part) CKC(cudaMalloc(&c->part, (size_t)wgrad_blocks() * kWgradRows * kWgradRow * 4));
+    // gradient of layer l's output lives in cur, with the layer's ReLU applied
+    // (layer 4 has none)
     const float *cur = dy;
     int slot = 0;
     for (int l = 4; l >= 1; --l) {
         const float *lin = l == 1 ? x : c->act[l - 1];
-        float *dmask = c->dbuf[slot];
-        if (l < 4) {
-            // cur already holds dL/d(out_l); apply the ReLU of layer l
-            relu_mask_kernel<<<device_sms() * 8, 256, 0, c->stream>>>(const_cast<float *>(cur), c->act[l], pix * c->ch[l]);
-            CKC(cudaGetLastError());
-        }
-        CKC(conv_wgrad_any(c->ch[l - 1], c->ch[l], lin, cur, c->g + c->woff[l], c->g + c->boff[l], N, H, W, c->stream));
+        float *dx = c->dbuf[slot];
+        CKC(conv_wgrad_any(c->ch[l - 1], c->ch[l], lin, cur, c->part, c->g + c->woff[l], N, H, W, c->stream));
         if (l > 1) {
-            transpose_flip_kernel<<<36, 256, 0, c->stream>>>(c->pb + c->woff[l], c->wt, c->ch[l], c->ch[l - 1]);
-            CKC(cudaGetLastError());
-            CKC(conv_fwd_any(c->ch[l], c->ch[l - 1], false, cur, c->wt, c->zero_bias, dmask, N, H, W, c->stream));
-            cur = dmask;
+            CKC(conv_dgrad_any(c->ch[l - 1], c->ch[l], cur, c->pb + c->woff[l], c->act[l - 1], dx, N, H, W, c->stream));
+            cur = dx;
             slot ^= 1;
         }
     }
