@@ -85,6 +85,8 @@ enum Ctr : int {
     kChanged = 3,        // cut extraction: a pass changed the set
     kStages = 4,         // ARD stages (low 32 bits; also kept in 64-bit below)
     kDischarges = 5,
+    kStop = 6,           // an earlier sweep of the window raised an error: discharge nothing
+    kTicket = 7,         // finished blocks of finish_flags_kernel
     kGlrFlags = 8,       // 3 words: global relabel "grew" flags
     kGlrLevels = 11,     // global relabel: levels run
     kCtrWords = 16
