@@ -324,16 +324,14 @@ __device__ __forceinline__ bool glr_level_block(const Geom &g, int W64, const Gl
     bool grew = false;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
-        if (yy[j] >= g.Y) continue;
-        Sout[(size_t)yy[j] * W64 + bx] = s[j];
+        const bool row = yy[j] < g.Y;
+        if (row) Sout[(size_t)yy[j] * W64 + bx] = s[j];
         // members found at this level get label max(d, level); level 0 changes nothing
-        u64 nw = level == 0 ? 0ull : (s[j] & ~s0[j]);
+        const u64 nw = level == 0 || !row ? 0ull : (s[j] & ~s0[j]);
         grew |= nw != 0ull;
-        for (; nw; nw &= nw - 1) {
-            const int x = bx * 64 + __ffsll((long long)nw) - 1;
-            int *p = &lab[(size_t)yy[j] * g.X + x];
-            if (*p < level) *p = level;
-        }
+        const size_t base = (size_t)yy[j] * g.X + (size_t)bx * 64;
+        raise_labels(lab, (unsigned)nw, base, level);
+        raise_labels(lab, (unsigned)(nw >> 32), base + 32, level);
     }
     return __any_sync(0xffffffffu, grew);
 }
@@ -856,6 +854,8 @@ GlrBatchBufs::~GlrBatchBufs() {
 bool glr2d_supported(const Geom &g) { return g.tz == 1 && g.Z == 1 && (g.tx == 64 || g.tx == 32); }
 
 cudaError_t glr2d(int conn, const Geom &g, const DevState &st, void *scratch, cudaStream_t s) {
+    // 32x32 tiles: a warp per region on 32-bit words (glr_stencil.cu)
+    if (stencil_glr_supported(conn, g)) return stencil_glr(conn, g, st, scratch, s);
     if (conn == 4) return glr2d_impl<4>(g, st, scratch, s);
     if (conn == 8) return glr2d_impl<8>(g, st, scratch, s);
     return cudaErrorInvalidValue;

@@ -38,21 +38,28 @@ __device__ __forceinline__ void glr3d_mask_row(const Geom &g, const DevState &st
     const size_t n = (size_t)g.n;
     const size_t nw = (size_t)g.Z * g.Y * W32;
     const size_t v0 = (size_t)row * g.X, w0 = (size_t)row * W32;
-    for (int xw = 0; xw < W32; ++xw) {
-        const int x = xw * 32 + lane;
-        const bool in = x < g.X;
-        const size_t v = v0 + x;
-        int c[6];
+    // two words of seven planes in flight; lane d stores the word of plane d
+    for (int xw = 0; xw < W32; xw += 2) {
+        int c[2][7];
 #pragma unroll
-        for (int d = 0; d < 6; ++d) c[d] = in ? __ldg(&st.cap[d * n + v]) : 0;
-        const int tc = in ? __ldg(&st.tcap[v]) : 0;
+        for (int u = 0; u < 2; ++u) {
+            const int x = (xw + u) * 32 + lane;
+            const bool in = x < g.X;
+            const size_t v = v0 + x;
 #pragma unroll
-        for (int d = 0; d < 6; ++d) {
-            const unsigned m = __ballot_sync(0xffffffffu, c[d] > 0);
-            if (lane == 0) M[d * nw + w0 + xw] = m;
+            for (int d = 0; d < 6; ++d) c[u][d] = in ? __ldg(&st.cap[d * n + v]) : 0;
+            c[u][6] = in ? __ldg(&st.tcap[v]) : 0;
         }
-        const unsigned m = __ballot_sync(0xffffffffu, tc > 0);
-        if (lane == 0) T[w0 + xw] = m;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            unsigned mine = 0;
+#pragma unroll
+            for (int d = 0; d < 7; ++d) {
+                const unsigned m = __ballot_sync(0xffffffffu, c[u][d] > 0);
+                if (lane == d) mine = m;
+            }
+            if (xw + u < W32 && lane < 7) (lane < 6 ? M + lane * nw : T)[w0 + xw + u] = mine;
+        }
     }
 }
 
@@ -159,17 +166,12 @@ __device__ bool glr3d_region(const Geom &g, int W32, int r, const u32 *__restric
     bool grew = false;
 #pragma unroll
     for (int j = 0; j < RPL; ++j) {
-        if (!rowin[j]) continue;
-        Sout[wi[j]] = s[j];
-        u32 nwb = level == 0 ? 0u : (s[j] & ~s0[j]);
+        if (rowin[j]) Sout[wi[j]] = s[j];
+        const u32 nwb = level == 0 || !rowin[j] ? 0u : (s[j] & ~s0[j]);
         grew |= nwb != 0u;
         if (!lab) continue;  // a plain closure: no labels
         const int rho = lane * RPL + j;
-        const size_t row0 = ((size_t)(rz * TZ + rho / TY) * g.Y + (ry * TY + rho % TY)) * g.X + (size_t)rx * 32;
-        for (; nwb; nwb &= nwb - 1) {
-            int *p = &lab[row0 + __ffs((int)nwb) - 1];
-            if (*p < level) *p = level;
-        }
+        raise_labels(lab, nwb, ((size_t)(rz * TZ + rho / TY) * g.Y + (ry * TY + rho % TY)) * g.X + (size_t)rx * 32, level);
     }
     return __any_sync(FULL, grew);
 }

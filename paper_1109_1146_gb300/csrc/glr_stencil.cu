@@ -1,6 +1,7 @@
-// Exact region-distance relabel (the global relabel heuristic) for the grids
-// with the longer displacements of the Sec. 7.1 synthetic networks, where the
-// bit-mask relabels (unit shifts) do not apply.
+// Exact region-distance relabel (the global relabel heuristic) for any 2D
+// stencil: the grids with the longer displacements of the Sec. 7.1 synthetic
+// networks, where the bit-mask relabel of cut2d.cu (unit shifts) does not apply,
+// and the 4- and 8-connected grids on 32x32 tiles.
 //
 // d*(u) = the least number of inter-region arcs on a residual path from u to
 // t (the region distance of Sec. 4.1, eq. 3).  Level sets S_0 ⊆ S_1 ⊆ ...:
@@ -16,7 +17,12 @@
 // tiles: one thread block per region, one byte per vertex in shared memory.
 // Bound by latency (grid barriers, L2 round trips).  500x500, connectivity 8,
 // 14 relabels of 26 levels: 54.6 ms as blocks on bytes with the capacities
-// read again in every pass, 4.9 ms as warps on masks.
+// read again in every pass, 4.9 ms as warps on masks (3.3 ms
+// with the labels of a row raised together).  Against the 64x64 blocks of
+// cut2d.cu (64-bit words, two rows per lane, every block at every level) on
+// 32x32 tiles: 1.02 -> 0.72 ms for the 7 relabels of the 637x419 8-connected
+// grid, 0.30 -> 0.22 ms (3, 1024x1024 4-connected), 0.89 -> 0.75 ms (3,
+// 2048x2048 8-connected).
 #include <algorithm>
 #include <climits>
 
@@ -277,15 +283,7 @@ __global__ void __launch_bounds__(128) stencil_glr_bits_kernel(const Geom g, con
                 sb.S[w] = S;
                 out[w] = joined;
             }
-            if (level > 0)
-                for (unsigned m = rows; m; m &= m - 1) {
-                    const int l = __ffs((int)m) - 1;
-                    const unsigned b = __shfl_sync(FULL, joined, l);
-                    const size_t v = (size_t)(ry * 32 + l) * g.X + rx * 32 + lane;
-                    if ((b >> lane) & 1u) {
-                        if (st.lab[v] < level) st.lab[v] = level;
-                    }
-                }
+            if (level > 0) raise_labels(st.lab, joined, (size_t)y * g.X + (size_t)rx * 32, level);
         }
         if (grew && lane == 0) atomicOr(&flags[level % 3], 1);
         if (blockIdx.x == 0 && threadIdx.x == 0) flags[(level + 1) % 3] = 0;
@@ -399,6 +397,7 @@ static cudaError_t stencil_glr_impl(const Geom &g, const DevState &st, void *scr
 }
 
 bool stencil_glr_supported(int conn, const Geom &g) {
+    if (conn == 4 || conn == 8) return g.tz == 1 && g.tx == 32 && g.ty == 32;  // called by glr2d for these tiles
     return is_paper(conn) && g.tz == 1 &&
            ((g.tx == 32 && g.ty == 32) || (conn == 108 && g.tx == 64 && (g.ty == 32 || g.ty == 64)));
 }
@@ -414,6 +413,8 @@ cudaError_t stencil_glr(int conn, const Geom &g, const DevState &st, void *scrat
         return g.ty == 64 ? stencil_glr_impl<108, 64, 64>(g, st, scratch, s) : stencil_glr_impl<108, 64, 32>(g, st, scratch, s);
     }
     switch (conn) {
+        case 4: return stencil_glr_bits<4>(g, st, scratch, s);
+        case 8: return stencil_glr_bits<8>(g, st, scratch, s);
         case 108: return stencil_glr_bits<108>(g, st, scratch, s);
         case 112: return stencil_glr_bits<112>(g, st, scratch, s);
         case 116: return stencil_glr_bits<116>(g, st, scratch, s);

@@ -1102,7 +1102,10 @@ mf_status mf_create_grid_ex(mf_grid **out, int ndim, const int64_t dims[3], int 
         {(void **)&g->st.left_active, (size_t)G.nreg}, {(void **)&g->st.flow_t, 8}, {(void **)&g->st.flow0, 8},
         {(void **)&g->st.hist, (kHistBins + 1) * 4}, {(void **)&g->st.ctr, kCtrWords * 4},
         {(void **)&g->smin, (size_t)n}, {(void **)&g->tset, (size_t)n}, {(void **)&g->c64, sizeof(Counters64)},
-        {(void **)&g->cut_scratch, paper ? stencil_glr_scratch_bytes(connectivity, G) : ndim == 2 ? cut2d_scratch_bytes(G, connectivity)
+        {(void **)&g->cut_scratch, paper ? stencil_glr_scratch_bytes(connectivity, G)
+                                   : ndim == 2 ? std::max(cut2d_scratch_bytes(G, connectivity),
+                                                          stencil_glr_supported(connectivity, G)
+                                                              ? stencil_glr_scratch_bytes(connectivity, G) : (size_t)0)
                                                        : (glr3d_supported(G) ? glr3d_scratch_bytes(G) : 0)}};
     for (auto &a : allocs) {
         if (a.bytes == 0) continue;

@@ -167,6 +167,32 @@ __device__ __forceinline__ void fence_proxy_async_smem() { asm volatile("fence.p
 #define DIAG_FLUSH() ((void)0)
 #endif
 
+// Labels of the vertices of up to 32 rows of 32, by one warp: lane l names row l's
+// vertices (bits) and where the row starts (base); every named label becomes
+// max(label, level).  A lane per column, so that a row's labels are one
+// coalesced access, four rows in flight (a lane per row took a round trip to
+// memory per vertex, up to 64 one after another).
+__device__ __forceinline__ void raise_labels(int *lab, unsigned bits, size_t base, int level) {
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned rows = __ballot_sync(kAll, bits != 0u);
+    while (rows) {
+        size_t o[4];
+        int v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int l = rows ? __ffs((int)rows) - 1 : 0;
+            const unsigned b = rows ? __shfl_sync(kAll, bits, l) : 0u;
+            o[q] = __shfl_sync(kAll, (unsigned long long)base, l) + lane;
+            rows &= rows - 1;
+            v[q] = (b >> lane) & 1u ? lab[o[q]] : kInf;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (v[q] < level) lab[o[q]] = level;
+    }
+}
+
 // one instance of a batch: its geometry, device state and statistics counters
 struct Inst {
     Geom g;
