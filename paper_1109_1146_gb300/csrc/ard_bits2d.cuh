@@ -1147,7 +1147,7 @@ __device__ __forceinline__ void discharge2d_region(const Geom &g, const DevState
 template <int CONN, int TX, int TY, int NT>
 __global__ void __launch_bounds__(NT, (Cfg2D<CONN, TX, TY, NT>::MINB)) ard_discharge2d_kernel(const Geom g, const DevState st, const SweepArgs sa) {
     const int r = blockIdx.x;
-    if (!st.active[r] || st.ctr[kStop]) return;
+    if (!region_to_discharge(st, r)) return;
     __shared__ __align__(8) unsigned long long s_mbar;
     if (threadIdx.x == 0) mbar_init(&s_mbar, 1);
     __syncthreads();

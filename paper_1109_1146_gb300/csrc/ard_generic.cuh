@@ -469,7 +469,7 @@ __device__ __forceinline__ void discharge_region(const Geom &g, const DevState &
 template <int CONN, int TX, int TY, int TZ, int NT>
 __global__ void __launch_bounds__(NT, 1) ard_discharge_kernel(const Geom g, const DevState st, const SweepArgs sa) {
     const int r = blockIdx.x;
-    if (!st.active[r] || st.ctr[kStop]) return;  // regions without active vertices are skipped (Sec. 5.3)
+    if (!region_to_discharge(st, r)) return;  // regions without active vertices are skipped (Sec. 5.3)
     discharge_region<CONN, TX, TY, TZ, NT>(g, st, sa, r);
 }
 

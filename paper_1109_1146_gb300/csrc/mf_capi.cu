@@ -309,90 +309,70 @@ __device__ __forceinline__ int hist_bin(int l) { return l < kHistBins ? l : kHis
 //   a refused push goes back to its sender (residual and excess restored).
 // Also commits the new boundary labels and keeps the histogram of boundary
 // labels (Sec. 5.3: the global gap needs labels of B only) up to date.
-// Fusion of one boundary vertex u = (lx, ly, lz) of region r at (rx, ry, rz)
-// (see above).  near: the discharged regions around r (region_flags).  The
-// boundary-label histogram change is returned as (old bin, new bin), -1 where
-// there is none, for the caller to aggregate over its warp.
+//
+// What fuse_arc does for u's arc d, whose head w lies in the region at offset
+// (qx, qy, qz); near: the discharged regions around u's (region_flags).
+// Returns whether u, below d_inf, received anything.
 template <int CONN>
-__device__ __forceinline__ void fuse_cell(const Geom &g, const DevState &st, const int rx, const int ry, const int rz,
-                                          const unsigned near, const int lx, const int ly, const int lz, int &bin_old,
-                                          int &bin_new) {
-    constexpr int N = arcs_of(CONN);
+__device__ __forceinline__ bool fuse_arc(const Geom &g, const DevState &st, const unsigned near, const int d,
+                                         const size_t u, const size_t w, const int qx, const int qy, const int qz) {
     const size_t n = (size_t)g.n;
-    const int x = rx * g.tx + lx, y = ry * g.ty + ly, z = rz * g.tz + lz;
+    const bool discr = (near >> kOwnRegion<CONN>) & 1u, discw = (near >> region_bit<CONN>(qx, qy, qz)) & 1u;
+    const int a = discr ? st.bout[(size_t)d * n + u] : 0, b = discw ? st.bout[(size_t)(d ^ 1) * n + w] : 0;
+    if (!(a | b)) return false;  // no flow crossed this arc: nothing to accept or return
+    const int du = discr ? st.lab_next[u] : st.lab[u], dw = discw ? st.lab_next[w] : st.lab[w];
+    const int back = (dw <= du + 1 ? 0 : a) + (du <= dw + 1 ? b : 0);
+    if (!back) return false;
+    st.cap[(size_t)d * n + u] += back;
+    atomicAdd(&st.exc[u], back);  // other arcs of u are other lanes' work
+    return du < g.dinf;
+}
+// the new label of the boundary vertex u of a discharged region; the histogram
+// change as (old bin, new bin), -1 where there is none
+__device__ __forceinline__ void commit_label(const Geom &g, const DevState &st, const size_t u, int &bin_old,
+                                             int &bin_new) {
+    const int old = st.lab[u], du = st.lab_next[u];
     bin_old = bin_new = -1;
-    if (!in_grid(g, x, y, z)) return;
-    const size_t u = ((size_t)z * g.Y + y) * g.X + x;
-    const bool discr = (near >> kOwnRegion<CONN>) & 1u;
-    // the flow over every crossing arc and u's labels: independent loads, one
-    // round trip (the Sec. 7.1 stencils have too many arcs to hold and take
-    // them one by one below)
-    int pu[is_paper(CONN) ? 1 : N], pw[is_paper(CONN) ? 1 : N];
-    bool boundary = false, flow = false;
-    auto load = [&](int d, int &a, int &b, size_t &w) {
-        const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d), wz = z + arc_dz(CONN, d);
-        a = b = 0;
-        w = 0;
-        if (!in_grid(g, wx, wy, wz)) return;
-        const int qx = (wx >> g.sx) - rx, qy = (wy >> g.sy) - ry, qz = (wz >> g.sz) - rz;
-        if (!(qx | qy | qz)) return;
-        boundary = true;
-        w = ((size_t)wz * g.Y + wy) * g.X + wx;
-        if (discr) a = st.bout[(size_t)d * n + u];
-        if ((near >> region_bit<CONN>(qx, qy, qz)) & 1u) b = st.bout[(size_t)(d ^ 1) * n + w];
-    };
-    if constexpr (!is_paper(CONN)) {
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-            size_t w;
-            load(d, pu[d], pw[d], w);
-        }
-    } else {
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-            const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d);
-            boundary |= wx >= 0 && wx < g.X && wy >= 0 && wy < g.Y && ((wx >> g.sx) != rx || (wy >> g.sy) != ry);
-        }
+    if (old == du) return;
+    if (old < g.dinf) bin_old = hist_bin(old);
+    if (du < g.dinf) bin_new = hist_bin(du);
+    st.lab[u] = du;
+}
+
+// The k-th cell of the tile whose arc d leaves the tile (4 / 8 / 6 stencils):
+// a face, or for a diagonal arc a row and a column.  False past the last.
+template <int CONN>
+__device__ __forceinline__ bool arc_cell(const Geom &g, const int d, const int k, int &lx, int &ly, int &lz) {
+    const int dx = arc_dx(CONN, d), dy = arc_dy(CONN, d), dz = arc_dz(CONN, d);
+    const int ex = dx > 0 ? g.tx - 1 : 0, ey = dy > 0 ? g.ty - 1 : 0, ez = dz > 0 ? g.tz - 1 : 0;
+    lz = 0;
+    if (dz) {
+        lx = k & (g.tx - 1);
+        ly = k >> g.sx;
+        lz = ez;
+        return k < g.tx * g.ty;
     }
-    if (!boundary) return;
-    const int old = st.lab[u];
-    const int du = discr ? st.lab_next[u] : old;
-    if constexpr (!is_paper(CONN)) {
-#pragma unroll
-        for (int d = 0; d < N; ++d) flow |= (pu[d] | pw[d]) != 0;
-    } else {
-        flow = true;
+    if (dx && dy) {
+        const bool row = k < g.tx;
+        lx = row ? k : ex;
+        ly = row ? ey : k - g.tx + (ey == 0);
+        return k < g.tx + g.ty - 1;
     }
-    if (flow) {  // else no flow crossed an arc of u: nothing to accept or return
-        int back_total = 0;
-#pragma unroll
-        for (int d = 0; d < N; ++d) {
-            int a, b;
-            if constexpr (is_paper(CONN)) {
-                size_t w;
-                load(d, a, b, w);
-            } else {
-                a = pu[d];
-                b = pw[d];
-            }
-            if (!(a | b)) continue;
-            const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d), wz = z + arc_dz(CONN, d);
-            const size_t w = ((size_t)wz * g.Y + wy) * g.X + wx;
-            const bool discw = (near >> region_bit<CONN>((wx >> g.sx) - rx, (wy >> g.sy) - ry, (wz >> g.sz) - rz)) & 1u;
-            const int dw = discw ? st.lab_next[w] : st.lab[w];
-            const int back = (dw <= du + 1 ? 0 : a) + (du <= dw + 1 ? b : 0);
-            if (back) {
-                st.cap[(size_t)d * n + u] += back;
-                back_total += back;
-            }
-        }
-        if (back_total) st.exc[u] += back_total;
+    if (dx) {
+        lx = ex;
+        ly = k & (g.ty - 1);
+        lz = k >> g.sy;
+        return k < g.ty * g.tz;
     }
-    if (discr && old != du) {
-        if (old < g.dinf) bin_old = hist_bin(old);
-        if (du < g.dinf) bin_new = hist_bin(du);
-        st.lab[u] = du;
-    }
+    lx = k & (g.tx - 1);
+    ly = ey;
+    lz = k >> g.sx;
+    return k < g.tx * g.tz;
+}
+template <int CONN>
+__device__ __forceinline__ int arc_cells(const Geom &g, const int d) {
+    const int dx = arc_dx(CONN, d), dy = arc_dy(CONN, d), dz = arc_dz(CONN, d);
+    return dz ? g.tx * g.ty : dx && dy ? g.tx + g.ty - 1 : dx ? g.ty * g.tz : g.tx * g.tz;
 }
 
 // Histogram updates of a warp: lanes naming the same bin send one atomic
@@ -448,117 +428,116 @@ __device__ __forceinline__ void surface_cell(const Geom &g, bool is3d, int p, in
     lz = 1 + q / (g.ty - 2);
 }
 
-// Fusion of one touched region over the tile surface (only surface cells can
-// be boundary vertices) by `split` warps, this one taking every split-th chunk
-// of 32 cells; returns whether the region was touched.
+// Fusion of one touched region by `split` warps, this one taking every split-th
+// chunk of 32 items: the surface cells' labels (if the region was discharged),
+// then the cells of every arc out of the tile that a discharge can have used.
+// The Sec. 7.1 stencils take the band cells with all their arcs instead.
+//
+// Activity: the discharge left 1 in left_active if a vertex below d_inf kept
+// excess; the fusion only adds excess, so beyond that a region is active iff a
+// vertex below d_inf received some, which is recorded as 2 (a region that was
+// not discharged had no active vertex).
 template <int CONN>
-__device__ __forceinline__ bool fuse_region_warp(const Geom &g, const DevState &st, const int r, const int part = 0,
+__device__ __forceinline__ void fuse_region_warp(const Geom &g, const DevState &st, const int r, const int part = 0,
                                                  const int split = 1) {
+    const int lane = threadIdx.x & 31;
     const int rx = r % g.RX, ry = (r / g.RX) % g.RY, rz = r / (g.RX * g.RY);
     const unsigned near = region_flags<CONN>(g, st, rx, ry, rz);
-    if (!near) return false;
-    // boundary vertices lie on the tile surface, or (the longer displacements
-    // of Sec. 7.1) anywhere in a band of the stencil's width: all cells then
-    const int P = is_paper(CONN) ? g.tx * g.ty : surface_cells(g, CONN == 6);
-    for (int p0 = part * 32; p0 < P; p0 += 32 * split) {  // whole warp per step: the histogram update is a warp operation
-        const int p = p0 + (threadIdx.x & 31);
-        int bo = -1, bn = -1;
-        if (p < P) {
-            int lx, ly, lz;
-            if (is_paper(CONN)) { lx = p & (g.tx - 1); ly = p >> g.sx; lz = 0; }
-            else surface_cell(g, CONN == 6, p, lx, ly, lz);
-            fuse_cell<CONN>(g, st, rx, ry, rz, near, lx, ly, lz, bo, bn);
+    if (!near) return;
+    const bool discr = (near >> kOwnRegion<CONN>) & 1u;
+    const int x0 = rx * g.tx, y0 = ry * g.ty, z0 = rz * g.tz;
+    bool act = false;
+    if constexpr (is_paper(CONN)) {
+        for (int p0 = part * 32; p0 < g.tx * g.ty; p0 += 32 * split) {  // whole warp per step: the histogram update is a warp operation
+            const int p = p0 + lane, x = x0 + (p & (g.tx - 1)), y = y0 + (p >> g.sx);
+            int bo = -1, bn = -1;
+            if (x < g.X && y < g.Y) {
+                const size_t u = (size_t)y * g.X + x;
+                bool boundary = false;
+#pragma unroll
+                for (int d = 0; d < arcs_of(CONN); ++d) {
+                    const int wx = x + arc_dx(CONN, d), wy = y + arc_dy(CONN, d);
+                    if (!in_grid(g, wx, wy, 0)) continue;
+                    const int qx = (wx >> g.sx) - rx, qy = (wy >> g.sy) - ry;
+                    if (!(qx | qy)) continue;
+                    boundary = true;
+                    act |= fuse_arc<CONN>(g, st, near, d, u, (size_t)wy * g.X + wx, qx, qy, 0);
+                }
+                if (boundary && discr) commit_label(g, st, u, bo, bn);
+            }
+            hist_update_warp(st.hist, bo, bn);
         }
-        hist_update_warp(st.hist, bo, bn);
+    } else {
+        int c = part;  // this warp's next chunk, counted from the current group of items
+        const int S = surface_cells(g, CONN == 6), LC = (S + 31) / 32;
+        if (discr)
+            for (; c < LC; c += split) {
+                const int p = c * 32 + lane;
+                int bo = -1, bn = -1, lx, ly, lz;
+                if (p < S) {
+                    surface_cell(g, CONN == 6, p, lx, ly, lz);
+                    const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+                    // (a surface cell at the border of the grid may have no neighbour region)
+                    const bool b = (lx == 0 && x > 0) || (lx == g.tx - 1 && x + 1 < g.X) || (ly == 0 && y > 0) ||
+                                   (ly == g.ty - 1 && y + 1 < g.Y) ||
+                                   (CONN == 6 && ((lz == 0 && z > 0) || (lz == g.tz - 1 && z + 1 < g.Z)));
+                    if (b && in_grid(g, x, y, z)) commit_label(g, st, ((size_t)z * g.Y + y) * g.X + x, bo, bn);
+                }
+                hist_update_warp(st.hist, bo, bn);
+            }
+        else
+            while (c < LC) c += split;
+        c -= LC;
+#pragma unroll
+        for (int d = 0; d < CONN; ++d) {
+            const int n = (arc_cells<CONN>(g, d) + 31) / 32;
+            const int dx = arc_dx(CONN, d), dy = arc_dy(CONN, d), dz = arc_dz(CONN, d);
+            // the regions the arc can lead to (a diagonal: three)
+            const bool used = discr || ((near >> region_bit<CONN>(dx, dy, dz)) & 1u) ||
+                              (dx && dy && ((near >> region_bit<CONN>(dx, 0, 0) | near >> region_bit<CONN>(0, dy, 0)) & 1u));
+            for (; c < n; c += split) {
+                int lx, ly, lz;
+                if (!used || !arc_cell<CONN>(g, d, c * 32 + lane, lx, ly, lz)) continue;
+                const int x = x0 + lx, y = y0 + ly, z = z0 + lz;
+                if (!in_grid(g, x, y, z) || !in_grid(g, x + dx, y + dy, z + dz)) continue;
+                const size_t u = ((size_t)z * g.Y + y) * g.X + x;
+                const size_t w = ((size_t)(z + dz) * g.Y + (y + dy)) * g.X + (x + dx);
+                act |= fuse_arc<CONN>(g, st, near, d, u, w, ((x + dx) >> g.sx) - rx, ((y + dy) >> g.sy) - ry,
+                                      ((z + dz) >> g.sz) - rz);
+            }
+            c -= n;
+        }
     }
-    return true;
+    if (__any_sync(0xffffffffu, act) && lane == 0) st.left_active[r] = st.left_active[r] | 2;
 }
 
-// Activity of one region after the fusion (one warp): with a gap, every label
-// g < d < d_inf of the tile becomes d_inf first (all cells); a touched region
-// is active if its discharge left interior excess (left_active) or a surface
-// vertex has excess below d_inf.
-// (PARTS: of `split` warps, each taking every split-th chunk of 32 cells; the
-// fusion has set active to left_active, a warp that finds an active vertex sets
-// it, and finish_flags_kernel counts)
-template <int CONN, bool PARTS>
-__device__ __forceinline__ void post_region_warp(const Geom &g, const DevState &st, const int r, const int gap,
-                                                 const int part = 0, const int split = 1) {
+// A gap (rare): every label g < d < d_inf of region r becomes d_inf, and whether
+// a border vertex of a touched region has excess below d_inf is found again
+// (one warp; 2 in left_active).
+template <int CONN>
+__device__ __forceinline__ void gap_region_warp(const Geom &g, const DevState &st, const int r, const int gap) {
     const int lane = threadIdx.x & 31;
     const int rx = r % g.RX, ry = (r / g.RX) % g.RY, rz = r / (g.RX * g.RY);
     const bool touched = region_flags<CONN>(g, st, rx, ry, rz) != 0;
-    if (!touched && gap == 0) return;
-    int act = touched && !PARTS ? st.left_active[r] : 0;
-    if (gap > 0) {
-        const int V = g.tx * g.ty * g.tz;
-        for (int i = part * 32 + lane; i < V; i += 32 * split) {
-            const int lx = i & (g.tx - 1), ly = (i >> g.sx) & (g.ty - 1), lz = i >> (g.sx + g.sy);
-            const int x = rx * g.tx + lx, y = ry * g.ty + ly, z = rz * g.tz + lz;
-            if (!in_grid(g, x, y, z)) continue;
-            const size_t u = ((size_t)z * g.Y + y) * g.X + x;
-            int l = st.lab[u];
-            if (l > gap && l < g.dinf) {
-                l = g.dinf;
-                st.lab[u] = l;
-            }
-            constexpr int R = radius_of(CONN);
-            const bool border = lx < R || lx >= g.tx - R || ly < R || ly >= g.ty - R ||
-                                (CONN == 6 && (lz == 0 || lz == g.tz - 1));
-            if (touched && border && l < g.dinf && st.exc[u] > 0) act = 1;
+    const int V = g.tx * g.ty * g.tz;
+    int act = 0;
+    for (int i = lane; i < V; i += 32) {
+        const int lx = i & (g.tx - 1), ly = (i >> g.sx) & (g.ty - 1), lz = i >> (g.sx + g.sy);
+        const int x = rx * g.tx + lx, y = ry * g.ty + ly, z = rz * g.tz + lz;
+        if (!in_grid(g, x, y, z)) continue;
+        const size_t u = ((size_t)z * g.Y + y) * g.X + x;
+        int l = st.lab[u];
+        if (l > gap && l < g.dinf) {
+            l = g.dinf;
+            st.lab[u] = l;
         }
-    } else {
-        const int P = is_paper(CONN) ? g.tx * g.ty : surface_cells(g, CONN == 6);
-        for (int p = part * 32 + lane; p < P && !act; p += 32 * split) {
-            int lx, ly, lz;
-            if (is_paper(CONN)) { lx = p & (g.tx - 1); ly = p >> g.sx; lz = 0; }
-            else surface_cell(g, CONN == 6, p, lx, ly, lz);
-            const int x = rx * g.tx + lx, y = ry * g.ty + ly, z = rz * g.tz + lz;
-            if (!in_grid(g, x, y, z)) continue;
-            const size_t u = ((size_t)z * g.Y + y) * g.X + x;
-            if (st.exc[u] > 0 && st.lab[u] < g.dinf) act = 1;
-        }
+        constexpr int R = radius_of(CONN);
+        const bool border = lx < R || lx >= g.tx - R || ly < R || ly >= g.ty - R ||
+                            (CONN == 6 && (lz == 0 || lz == g.tz - 1));
+        if (touched && border && l < g.dinf && st.exc[u] > 0) act = 1;
     }
     act = __any_sync(0xffffffffu, act);
-    if (lane == 0 && touched) {
-        if (PARTS) {
-            if (act) st.active[r] = 1;
-            return;
-        }
-        st.active[r] = (unsigned char)act;
-        if (act) atomicAdd(&st.ctr[kActiveRegions], 1);
-    }
-}
-
-// single grid: `split` warps per region, grid-stride.  A region is a chain of
-// dependent loads per chunk of 32 surface cells (4 chunks in a 32x32 tile, 21 in
-// 32x8x4, 32 for the Sec. 7.1 stencils), so a grid with fewer regions than the
-// chip holds warps spreads the chunks over them; with more regions one warp each
-// is cheaper (the test whether a region was touched is made once).
-static int surface_split(const Geom &g, int conn) {
-    const int cells = is_paper(conn) ? g.tx * g.ty
-                      : conn == 6 ? 2 * g.tx * g.ty + 2 * g.tx * (g.tz - 2) + 2 * (g.ty - 2) * (g.tz - 2)
-                                  : 2 * g.tx + 2 * (g.ty - 2);
-    return std::max(1, std::min((cells + 31) / 32, device_sms() * 64 / g.nreg));
-}
-template <int CONN>
-__global__ void fuse_warp_kernel(const Geom g, const DevState st, const int split) {
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    const int items = g.nreg * split;  // (split > 1 only below the number of warps the chip holds)
-    for (int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < items; k += nw) {
-        const int r = split == 1 ? k : k / split, part = k - r * split;
-        if (fuse_region_warp<CONN>(g, st, r, part, split) && part == 0 && (threadIdx.x & 31) == 0)
-            st.active[r] = st.left_active[r];
-    }
-}
-template <int CONN>
-__global__ void post_warp_kernel(const Geom g, const DevState st, const int split) {
-    const int gap = st.ctr[kGap];
-    const int nw = gridDim.x * (blockDim.x >> 5);
-    const int items = g.nreg * split;
-    for (int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < items; k += nw) {
-        const int r = split == 1 ? k : k / split;
-        post_region_warp<CONN, true>(g, st, r, gap, k - r * split, split);
-    }
+    if (lane == 0 && touched) st.left_active[r] = (unsigned char)((st.left_active[r] & 1) | (act ? 2 : 0));
 }
 
 // Global gap (Sec. 5.1, with the boundary-label histogram of Sec. 5.3): the
@@ -571,13 +550,13 @@ __device__ __forceinline__ void gap_find_body(const DevState &st) {
     __syncthreads();
     int hi = 0;
     for (int b = threadIdx.x; b <= kHistBins; b += blockDim.x)
-        if (st.hist[b] > 0) hi = max(hi, b);
+        if (__ldcg(&st.hist[b]) > 0) hi = max(hi, b);
     atomicMax(&s_hi, hi);
     __syncthreads();
     const int top = s_hi;  // labels >= kHistBins share the last bin: never a gap there
     int gmin = INT_MAX;
     for (int b = 1 + threadIdx.x; b < top && b < kHistBins; b += blockDim.x)
-        if (st.hist[b] == 0) gmin = min(gmin, b);
+        if (__ldcg(&st.hist[b]) == 0) gmin = min(gmin, b);
     atomicMin(&s_g, gmin);
     __syncthreads();
     const int gap = s_g == INT_MAX ? 0 : s_g;
@@ -586,28 +565,77 @@ __device__ __forceinline__ void gap_find_body(const DevState &st) {
         for (int b = gap + 1 + threadIdx.x; b <= kHistBins; b += blockDim.x) st.hist[b] = 0;
 }
 
-__global__ void gap_find_kernel(const DevState st) { gap_find_body(st); }
-
-// Count the active regions, reset the per-sweep flags.  With a log (a pinned
-// record of the sweep: active regions, error, gap) the last block to finish
-// writes it, makes later sweeps of the window discharge nothing after an error,
-// and clears the counters for the next sweep.
-__global__ void finish_flags_kernel(const DevState st, int nreg, int4 *log) {
-    int c = 0;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < nreg; r += gridDim.x * blockDim.x) {
-        c += st.active[r] != 0;
-        st.disc[r] = 0;
-        st.left_active[r] = 0;
+// single grid: `split` warps per region, grid-stride.  A region is a chain of
+// dependent loads per chunk of 32 items (8 chunks in a 4-connected 32x32 tile, 47
+// in 32x8x4, 32 for the Sec. 7.1 stencils), so a grid with fewer regions than
+// the chip holds warps spreads the chunks over them; with more regions one warp
+// each is cheaper (the flags around a region are read once).
+static int surface_split(const Geom &g, int conn) {
+    const int surface = conn == 6 ? 2 * (g.tx * g.ty + g.tx * g.tz + g.ty * g.tz) : 2 * (g.tx + g.ty);
+    const int chunks = is_paper(conn) ? g.tx * g.ty / 32 : (surface + (conn == 8 ? 2 * surface : surface)) / 32;
+    return std::max(1, std::min(chunks, device_sms() * 64 / g.nreg));
+}
+// Fusion; with gap_on the last block to finish also looks for the global gap
+// (a kernel of its own cost 5 us and a launch).
+template <int CONN>
+__global__ void __launch_bounds__(256) fuse_warp_kernel(const Geom g, const DevState st, const int split, const bool gap_on) {
+    if (st.ctr[kStop]) return;
+    const int nw = gridDim.x * (blockDim.x >> 5);
+    const int items = g.nreg * split;  // (split > 1 only below the number of warps the chip holds)
+    for (int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < items; k += nw) {
+        const int r = split == 1 ? k : k / split;
+        fuse_region_warp<CONN>(g, st, r, k - r * split, split);
     }
-    c = __reduce_add_sync(0xffffffffu, c);
-    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&st.ctr[kActiveRegions], c);
+    if (!gap_on) return;
+    __shared__ bool s_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = atomicAdd(&st.ctr[kTicket], 1) == (int)gridDim.x - 1;
+        if (s_last) st.ctr[kTicket] = 0;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    gap_find_body(st);
+}
+
+// Activity of every region for the next sweep (after a gap: the labels first)
+// and the number of active regions.  With a log (a pinned record of the sweep:
+// active regions, error, gap) the last block to finish writes it, makes later
+// sweeps of the window do nothing after an error, and clears the counters for
+// the next sweep.
+template <int CONN>
+__global__ void __launch_bounds__(256) finish_sweep_kernel(const Geom g, const DevState st, int4 *log) {
+    if (st.ctr[kStop]) return;
+    const int gap = st.ctr[kGap];
+    if (gap > 0) {
+        const int nw = gridDim.x * (blockDim.x >> 5);
+        for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < g.nreg; r += nw) {
+            gap_region_warp<CONN>(g, st, r, gap);
+            if ((threadIdx.x & 31) == 0) {
+                const bool act = st.left_active[r] != 0;
+                st.active[r] = act;
+                if (act) atomicAdd(&st.ctr[kActiveRegions], 1);
+            }
+        }
+    } else {
+        int c = 0;
+        for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < g.nreg; r += gridDim.x * blockDim.x) {
+            const bool act = st.left_active[r] != 0;
+            st.active[r] = act;
+            c += act;
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        if ((threadIdx.x & 31) == 0 && c) atomicAdd(&st.ctr[kActiveRegions], c);
+    }
     if (!log) return;
     __threadfence();
     __syncthreads();
     if (threadIdx.x != 0 || atomicAdd(&st.ctr[kTicket], 1) != (int)gridDim.x - 1) return;
     __threadfence();
     const int active = atomicExch(&st.ctr[kActiveRegions], 0), error = atomicExch(&st.ctr[kError], 0);
-    *log = make_int4(active, error, st.ctr[kGap], 0);
+    *log = make_int4(active, error, gap, 0);
     if (error) st.ctr[kStop] = 1;
     st.ctr[kTicket] = 0;
 }
@@ -693,27 +721,47 @@ __global__ void fuse_batch_kernel(const Inst *insts, const int2 *regs, int nregs
     }
 }
 
-__global__ void gap_find_batch_kernel(const Inst *insts, const unsigned char *done) {
+__global__ void gap_find_batch_kernel(const Inst *insts, const unsigned char *done, int *any_gap) {
     if (done[blockIdx.x]) return;
     gap_find_body(insts[blockIdx.x].st);
+    __syncthreads();
+    if (threadIdx.x == 0 && insts[blockIdx.x].st.ctr[kGap] > 0) *any_gap = 1;
 }
 
+// the labels of the instances that found a gap in this sweep
 template <int CONN>
-__global__ void post_batch_kernel(const Inst *insts, const int2 *regs, int nregs, const unsigned char *done) {
+__global__ void gap_batch_kernel(const Inst *insts, const int2 *regs, int nregs, const unsigned char *done,
+                                 const int *any_gap) {
+    if (!*any_gap) return;
     const int nw = gridDim.x * (blockDim.x >> 5);
     for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < nregs; i += nw) {
         const int2 w = regs[i];
         if (done[w.x] || insts[w.x].conn != CONN) continue;
-        post_region_warp<CONN, false>(insts[w.x].g, insts[w.x].st, w.y, insts[w.x].st.ctr[kGap]);
+        const int gap = insts[w.x].st.ctr[kGap];
+        if (gap > 0) gap_region_warp<CONN>(insts[w.x].g, insts[w.x].st, w.y, gap);
     }
 }
 
-__global__ void clear_batch_kernel(const Inst *insts, const int2 *regs, int nregs, const unsigned char *done) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nregs; i += gridDim.x * blockDim.x) {
-        const int2 w = regs[i];
-        if (done[w.x]) continue;
-        insts[w.x].st.disc[w.y] = 0;
-        insts[w.x].st.left_active[w.y] = 0;
+// activity of every region and the active regions of every instance (one atomic
+// per instance and warp); the per-sweep flags are cleared
+__global__ void finish_batch_kernel(const Inst *insts, const int2 *regs, int nregs, const unsigned char *done) {
+    const int lane = threadIdx.x & 31;
+    for (int i0 = blockIdx.x * blockDim.x + (threadIdx.x - lane); i0 < nregs; i0 += gridDim.x * blockDim.x) {
+        const int i = i0 + lane;
+        int key = -1;
+        if (i < nregs) {
+            const int2 w = regs[i];
+            if (!done[w.x]) {
+                const DevState &st = insts[w.x].st;
+                const bool act = st.left_active[w.y] != 0;
+                st.active[w.y] = act;
+                st.disc[w.y] = 0;
+                st.left_active[w.y] = 0;
+                if (act) key = w.x;
+            }
+        }
+        const unsigned m = __match_any_sync(0xffffffffu, key);
+        if (key >= 0 && lane == __ffs(m) - 1) atomicAdd(&insts[key].st.ctr[kActiveRegions], __popc(m));
     }
 }
 
@@ -845,10 +893,9 @@ template <int CONN>
 static cudaError_t launch_fuse_post(mf_grid *h, bool gap_on, cudaStream_t st, int4 *log = nullptr) {
     const int split = surface_split(h->g, CONN);
     const int wb = (int)std::min<long long>(((long long)h->g.nreg * split + 7) / 8, (long long)device_sms() * 8);
-    fuse_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st, split);
-    if (gap_on) gap_find_kernel<<<1, 1024, 0, st>>>(h->st);
-    post_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st, split);
-    finish_flags_kernel<<<(h->g.nreg + 255) / 256, 256, 0, st>>>(h->st, h->g.nreg, log);
+    fuse_warp_kernel<CONN><<<wb, 256, 0, st>>>(h->g, h->st, split, gap_on);
+    const int fb = (int)std::min<long long>(((long long)h->g.nreg + 7) / 8, (long long)device_sms());
+    finish_sweep_kernel<CONN><<<fb, 256, 0, st>>>(h->g, h->st, log);
     return cudaGetLastError();
 }
 template <int CONN>
@@ -1580,7 +1627,7 @@ static mf_status run_window(mf_grid *g, int count, bool defer, int32_t *active_o
         CK(cudaEventRecord(g->wev[3 * i + 1], g->stream));
         CK(DISPATCH(g->conn, launch_fuse_post, g, g->opts.global_gap != 0, g->stream, g->h_log_dv + i));
         CK(cudaEventRecord(g->wev[3 * i + 2], g->stream));
-        g->launches += g->opts.global_gap ? 5 : 4;
+        g->launches += 3;  // discharge, fusion, finish
     }
     CK(cudaStreamSynchronize(g->stream));
     // the previous window's relabel: with no region active after it there was
@@ -1794,7 +1841,7 @@ static mf_status run_graph_loop(mf_grid *g, long long cap) {
     init[kLoopFirst] = glr_supported(g) ? std::max(0, g->opts.global_relabel_first) : 0;
     memcpy(g->h_loop, init, sizeof(init));
     CK(cudaMemcpyAsync(g->loopctl, g->h_loop, kLoopWords * 4, cudaMemcpyHostToDevice, g->stream));
-    const int per_sweep = g->opts.global_gap ? 6 : 5;
+    const int per_sweep = 4;  // discharge, fusion, finish, loop control
     for (;;) {
         const int before = g->sweep;
         CK(cudaGraphLaunch(g->graph_exec, g->stream));
@@ -2072,7 +2119,7 @@ mf_status mf_solve_batch(mf_grid *const *grids, int count, const mf_opts *opts, 
     CK(cudaMalloc(&B.cnt, sizeof(int) * nt));
     CK(cudaMalloc(&B.head, sizeof(int) * nt));
     CK(cudaMalloc(&B.sweeps, sizeof(int) * count));
-    CK(cudaMalloc(&B.any, sizeof(int)));
+    CK(cudaMalloc(&B.any, 2 * sizeof(int)));  // instances still active; some instance found a gap
     CK(cudaMalloc(&B.done, count));
     CK(cudaMemcpyAsync(B.insts, hinst.data(), sizeof(Inst) * count, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(B.regs, hregs.data(), sizeof(int2) * nregs, cudaMemcpyHostToDevice, s));
@@ -2088,7 +2135,14 @@ mf_status mf_solve_batch(mf_grid *const *grids, int count, const mf_opts *opts, 
     const int wbb = (int)std::min<long long>(((long long)nregs + 7) / 8, (long long)device_sms() * 8);
     mf_status rs = MF_OK;
     long long launches = 0;
-    const int per_sweep = 6 + nt + (o.global_gap ? 1 : 0);
+    int nconn = 0;  // connectivities present
+    for (int conn : {4, 8, 6}) {
+        bool has = false;
+        for (auto &ty : types) has |= ty.conn == conn;
+        nconn += has;
+    }
+    // resets, work lists, discharges, fusions, finish, end; with the gap: its search and the labels
+    const int per_sweep = 4 + nt + nconn + (o.global_gap ? 1 + nconn : 0);
     // host loop: the persistent discharge launches of each kernel type are
     // timed with events (no event can be recorded inside the graph's loop body)
     std::vector<double> type_ms(nt, 0.0);
@@ -2106,7 +2160,7 @@ mf_status mf_solve_batch(mf_grid *const *grids, int count, const mf_opts *opts, 
         a.sweep_dev = sweep_dev;
         cudaError_t e = cudaMemsetAsync(B.cnt, 0, sizeof(int) * nt, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(B.head, 0, sizeof(int) * nt, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(B.any, 0, sizeof(int), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(B.any, 0, 2 * sizeof(int), st);
         if (e != cudaSuccess) return e;
         batch_reset_kernel<<<(count + 255) / 256, 256, 0, st>>>(B.insts, B.done, count);
         batch_items_kernel<<<eb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done, B.type_of, nregs, B.items, B.cnt);
@@ -2129,16 +2183,18 @@ mf_status mf_solve_batch(mf_grid *const *grids, int count, const mf_opts *opts, 
             if (conn == 8) fuse_batch_kernel<8><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
             if (conn == 6) fuse_batch_kernel<6><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
         }
-        if (o.global_gap) gap_find_batch_kernel<<<count, 1024, 0, st>>>(B.insts, B.done);
-        for (int conn : {4, 8, 6}) {
-            bool has = false;
-            for (auto &ty : types) has |= ty.conn == conn;
-            if (!has) continue;
-            if (conn == 4) post_batch_kernel<4><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
-            if (conn == 8) post_batch_kernel<8><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
-            if (conn == 6) post_batch_kernel<6><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
+        if (o.global_gap) {
+            gap_find_batch_kernel<<<count, 1024, 0, st>>>(B.insts, B.done, B.any + 1);
+            for (int conn : {4, 8, 6}) {
+                bool has = false;
+                for (auto &ty : types) has |= ty.conn == conn;
+                if (!has) continue;
+                if (conn == 4) gap_batch_kernel<4><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done, B.any + 1);
+                if (conn == 8) gap_batch_kernel<8><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done, B.any + 1);
+                if (conn == 6) gap_batch_kernel<6><<<wbb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done, B.any + 1);
+            }
         }
-        clear_batch_kernel<<<eb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
+        finish_batch_kernel<<<eb, 256, 0, st>>>(B.insts, B.regs, nregs, B.done);
         batch_end_kernel<<<(count + 255) / 256, 256, 0, st>>>(B.insts, B.done, B.sweeps, B.any, count);
         return cudaGetLastError();
     };

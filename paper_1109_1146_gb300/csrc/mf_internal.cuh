@@ -104,6 +104,18 @@ struct SweepArgs {
     Counters64 *c64;
 };
 
+// Has region r, the block's, to be discharged in this sweep?  A region that has
+// not clears its flags of the sweep before (after an error nothing is touched).
+__device__ __forceinline__ bool region_to_discharge(const DevState &st, int r) {
+    const bool stop = st.ctr[kStop] != 0, active = st.active[r] != 0;
+    if (active && !stop) return true;
+    if (threadIdx.x == 0 && !stop) {
+        st.disc[r] = 0;
+        st.left_active[r] = 0;
+    }
+    return false;
+}
+
 // ---- bulk asynchronous copies (TMA engine, no tensor map) into shared memory
 // A transaction barrier (mbarrier) in shared memory counts the bytes of the
 // copies issued against it; the phase completes when they have all landed.
