@@ -48,7 +48,8 @@ namespace mf {
 #define mf_diag mf_diag3
 #endif
 
-template <int TY, int TZ, int NT>
+// MB: resident blocks per SM the registers must allow
+template <int TY, int TZ, int NT, int MB>
 struct Cfg3D {
     static constexpr int TX = 32, N = 6;
     static constexpr int NR = TY * TZ;            // rows of the tile
@@ -61,15 +62,12 @@ struct Cfg3D {
     static constexpr int B_MX = 0, B_PX = NR, B_MY = 2 * NR, B_PY = 2 * NR + TX * TZ;
     static constexpr int B_MZ = 2 * NR + 2 * TX * TZ, B_PZ = B_MZ + TX * TY;
     static constexpr int HL = B_PZ + TX * TY;     // halo cells = arcs leaving the tile
-    static constexpr int LCAP = 32;               // BFS layers kept as masks
-    // resident blocks per SM the registers must allow (shared memory allows
-    // eight 16-row tiles at 128 threads, four 32x8x4 tiles, two 32x8x8 tiles,
-    // one 32x16x8 tile)
-    static constexpr int MINB = NR == 16 ? 8 : NR == 32 ? 4 : NR == 64 ? 2 : 1;
+    // BFS layers kept as masks (24 let five 32x8x4 tiles share an SM's memory)
+    static constexpr int LCAP = MB == 5 ? 24 : 32;
     static constexpr size_t smem = (size_t)(N + 3) * V * 4           // cap, tcap, exc, lab
                                    + (size_t)(N + 4) * NR * 4        // R[N], T, E, inc, vis
                                    + (size_t)(LCAP + 1) * NR * 4     // BFS layers 1..LCAP
-                                   + (size_t)2 * HL * 4 + NR + 16;   // halo labels, hm, dirty rows, padding
+                                   + (size_t)HL * 4 + NR + 16;       // halo labels, dirty rows, padding
     // after this many passes of the graph warp over a push layer the rest of it
     // is handed to all warps
     static constexpr int HEAVY = 8;
@@ -171,12 +169,14 @@ __device__ __forceinline__ void send_arcs3(unsigned a, const int (&c)[sizeof...(
 // and 5-6 push layers per discharge).  By all warps, a row per warp with a
 // block barrier per layer and the masks rebuilt after a round, a push layer took
 // 2100-2400 cycles and a BFS layer 320-350, now 1000 and 95.  Discharge time of a
-// solve: 382 -> 209 ms (512x512x384), 12.4 -> 6.9 ms (128^3), 6.1 -> 3.5 ms
-// (61x75x53).
-template <int TY, int TZ, int NT>
+// solve: 382 -> 181 ms (512x512x384), 12.4 -> 6.7 ms (128^3), 6.1 -> 3.4 ms
+// (61x75x53).  128 threads per 32x8x4 region in single solves (the graph warp
+// without register spills: 210 -> 203 ms on 512x512x384), 256 in batches (62
+// against 65 ms for the batch of 48 2D and 16 3D grids).
+template <int TY, int TZ, int NT, int MB>
 __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState &st, const SweepArgs &sa,
                                                    const int r, unsigned long long *mbar, unsigned &mphase) {
-    using C = Cfg3D<TY, TZ, NT>;
+    using C = Cfg3D<TY, TZ, NT, MB>;
     constexpr int TX = 32, N = 6, V = C::V, NR = C::NR, RPL = C::RPL, NW = C::NW, LCAP = C::LCAP, LZ = C::LZ;
     constexpr unsigned FULL = 0xffffffffu;
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -192,9 +192,8 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     u32 *s_vis = s_inc + NR;                // [NR] final closure (during Augment rounds: excess received)
     u32 *s_layer = s_vis + NR;              // [LCAP+1][NR]
     int *s_hl = (int *)(s_layer + (LCAP + 1) * NR);  // [HL] labels of B^R
-    int *s_hm = s_hl + C::HL;               // [HL] label of the halo cell if its arc is residual, else INT_MAX
     // [NR] rows whose planes changed (2: by the current command's pushes)
-    unsigned char *s_dirty = (unsigned char *)(s_hm + C::HL);
+    unsigned char *s_dirty = (unsigned char *)(s_hl + C::HL);
     __shared__ int s_ctl[5];                // command, its argument, epoch, any augmentation, stage
     __shared__ unsigned long long s_flow;
     enum { kDone = 0, kLabel = 1, kPush = 2 };
@@ -287,11 +286,6 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     }
     __syncthreads();
     for (int rho = warp; rho < NR; rho += NW) rebuild_row(rho);
-    for (int h = tid; h < C::HL; h += NT) {
-        int lx, ly, lz, d;
-        halo3_src<TY, TZ>(h, lx, ly, lz, d);
-        s_hm[h] = s_cap[d * V + (lz * TY + ly) * TX + lx] > 0 ? s_hl[h] : INT_MAX;
-    }
     __syncthreads();
     DIAG_LAP(0);
 
@@ -318,39 +312,41 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
         }
         return __reduce_min_sync(FULL, best);
     };
-    // boundary part of the seed rows of T_k: a residual arc to a halo cell w with d(w) < k
+    // boundary part of the seed rows of T_k: a residual arc to a halo cell w with
+    // d(w) < k.  The masks of arcs that leave the tile stay in s_R (push_out
+    // keeps them up to date).
     auto seed_boundary = [&](int k) {
+        u32 my[RPL], py[RPL], mz[RPL], pz[RPL];
 #pragma unroll
         for (int j = 0; j < RPL; ++j) {
             const int rho = lane * RPL + j;
             u32 s = 0u;
+            my[j] = py[j] = mz[j] = pz[j] = 0u;
             if (lrow) {
-                if (s_hm[C::B_MX + rho] < k) s |= 1u;
-                if (s_hm[C::B_PX + rho] < k) s |= 1u << (TX - 1);
+                if (s_hl[C::B_MX + rho] < k) s |= s_R[1 * NR + rho] & 1u;
+                if (s_hl[C::B_PX + rho] < k) s |= s_R[rho] & (1u << (TX - 1));
+                py[j] = row_has(2, rho) ? 0u : s_R[2 * NR + rho];
+                my[j] = row_has(3, rho) ? 0u : s_R[3 * NR + rho];
+                pz[j] = row_has(4, rho) ? 0u : s_R[4 * NR + rho];
+                mz[j] = row_has(5, rho) ? 0u : s_R[5 * NR + rho];
             }
             sdB[j] = s;
         }
 #pragma unroll
         for (int z = 0; z < TZ; ++z) {
-            const u32 bm = __ballot_sync(FULL, s_hm[C::B_MY + z * TX + lane] < k);
-            const u32 bp = __ballot_sync(FULL, s_hm[C::B_PY + z * TX + lane] < k);
+            const u32 bm = __ballot_sync(FULL, s_hl[C::B_MY + z * TX + lane] < k);
+            const u32 bp = __ballot_sync(FULL, s_hl[C::B_PY + z * TX + lane] < k);
 #pragma unroll
-            for (int j = 0; j < RPL; ++j) {
-                const int rho = lane * RPL + j;
-                if (rho == z * TY) sdB[j] |= bm;
-                if (rho == z * TY + TY - 1) sdB[j] |= bp;
-            }
+            for (int j = 0; j < RPL; ++j)
+                if ((lane * RPL + j) / TY == z) sdB[j] |= (bm & my[j]) | (bp & py[j]);
         }
 #pragma unroll
         for (int y = 0; y < TY; ++y) {
-            const u32 bm = __ballot_sync(FULL, s_hm[C::B_MZ + y * TX + lane] < k);
-            const u32 bp = __ballot_sync(FULL, s_hm[C::B_PZ + y * TX + lane] < k);
+            const u32 bm = __ballot_sync(FULL, s_hl[C::B_MZ + y * TX + lane] < k);
+            const u32 bp = __ballot_sync(FULL, s_hl[C::B_PZ + y * TX + lane] < k);
 #pragma unroll
-            for (int j = 0; j < RPL; ++j) {
-                const int rho = lane * RPL + j;
-                if (rho == y) sdB[j] |= bm;
-                if (rho == (TZ - 1) * TY + y) sdB[j] |= bp;
-            }
+            for (int j = 0; j < RPL; ++j)
+                if ((lane * RPL + j) % TY == y) sdB[j] |= (bm & mz[j]) | (bp & pz[j]);
         }
     };
     // the words of the rows one step along each arc direction (2..5) from the
@@ -430,7 +426,7 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     long long flow_acc = 0;
     // what the vertex at column x of row rho with excess e, in layer 1, sends
     // into B^R; returns the rest.  seed: has it still a residual arc into T_k's
-    // boundary vertices (s_hm is kept up to date)
+    // boundary vertices
     auto push_out = [&](int x, int rho, int e, int k, bool &seed) -> int {
         const int ly = rho % TY, lz = rho / TY, i = rho * TX + x;
         seed = false;
@@ -443,7 +439,7 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
                 const int b = min(e, c);
                 s_cap[d * V + i] = c - b;
                 e -= b;
-                if (b == c) s_hm[h] = INT_MAX;
+                if (b == c) atomicAnd(&s_R[d * NR + rho], ~(1u << x));
                 else seed = true;
             }
         }
@@ -994,19 +990,19 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
     }
 }
 
-template <int TY, int TZ, int NT>
-__global__ void __launch_bounds__(NT, (Cfg3D<TY, TZ, NT>::MINB)) ard_discharge3d_kernel(const Geom g, const DevState st, const SweepArgs sa) {
+template <int TY, int TZ, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) ard_discharge3d_kernel(const Geom g, const DevState st, const SweepArgs sa) {
     const int r = blockIdx.x;
     if (!region_to_discharge(st, r)) return;
     __shared__ __align__(8) unsigned long long s_mbar;
     if (threadIdx.x == 0) mbar_init(&s_mbar, 1);
     __syncthreads();
     unsigned phase = 0;
-    discharge3d_region<TY, TZ, NT>(g, st, sa, r, &s_mbar, phase);
+    discharge3d_region<TY, TZ, NT, MB>(g, st, sa, r, &s_mbar, phase);
 }
 
-template <int TY, int TZ, int NT>
-__global__ void __launch_bounds__(NT, (Cfg3D<TY, TZ, NT>::MINB))
+template <int TY, int TZ, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB)
 ard_discharge3d_batch_kernel(const Inst *__restrict__ insts, const int2 *__restrict__ items, const int *count,
                              int *head, const SweepArgs sa) {
     __shared__ int s_it;
@@ -1023,14 +1019,14 @@ ard_discharge3d_batch_kernel(const Inst *__restrict__ insts, const int2 *__restr
         const Inst &I = insts[w.x];
         SweepArgs a = sa;
         a.c64 = I.c64;
-        discharge3d_region<TY, TZ, NT>(I.g, I.st, a, w.y, &s_mbar, phase);
+        discharge3d_region<TY, TZ, NT, MB>(I.g, I.st, a, w.y, &s_mbar, phase);
     }
 }
 
-template <int TY, int TZ, int NT>
+template <int TY, int TZ, int NT, int MB>
 static cudaError_t launch3d(const Geom &g, const DevState &st, const SweepArgs &sa, cudaStream_t s) {
-    using C = Cfg3D<TY, TZ, NT>;
-    auto k = ard_discharge3d_kernel<TY, TZ, NT>;
+    using C = Cfg3D<TY, TZ, NT, MB>;
+    auto k = ard_discharge3d_kernel<TY, TZ, NT, MB>;
     {
         const cudaError_t e_at = ensure_smem_attr((const void *)k, (int)C::smem);
         if (e_at != cudaSuccess) return e_at;
@@ -1039,17 +1035,17 @@ static cudaError_t launch3d(const Geom &g, const DevState &st, const SweepArgs &
     return cudaGetLastError();
 }
 
-template <int TY, int TZ, int NT>
+template <int TY, int TZ, int NT, int MB>
 static cudaError_t launch3d_batch(const Inst *insts, const int2 *items, const int *count, int *head,
                                   const SweepArgs &sa, int blocks, cudaStream_t s) {
-    using C = Cfg3D<TY, TZ, NT>;
-    auto k = ard_discharge3d_batch_kernel<TY, TZ, NT>;
+    using C = Cfg3D<TY, TZ, NT, MB>;
+    auto k = ard_discharge3d_batch_kernel<TY, TZ, NT, MB>;
     {
         const cudaError_t e_at = ensure_smem_attr((const void *)k, (int)C::smem);
         if (e_at != cudaSuccess) return e_at;
     }
     // persistent blocks: at least as many as can be resident
-    const int resident = device_sms() * C::MINB;
+    const int resident = device_sms() * MB;
     k<<<blocks > resident ? blocks : resident, NT, C::smem, s>>>(insts, items, count, head, sa);
     return cudaGetLastError();
 }
@@ -1059,22 +1055,33 @@ bool discharge3d_supported(int tx, int ty, int tz) {
                         (ty == 8 && tz == 2));
 }
 
+constexpr int kMany3d = 48;  // active regions per SM from which five are resident
+
 cudaError_t launch_discharge3d(const Geom &g, const DevState &st, const SweepArgs &sa, cudaStream_t stream) {
-    if (g.tx == 32 && g.ty == 16 && g.tz == 8) return launch3d<16, 8, 512>(g, st, sa, stream);
-    if (g.tx == 32 && g.ty == 8 && g.tz == 8) return launch3d<8, 8, 256>(g, st, sa, stream);
-    if (g.tx == 32 && g.ty == 8 && g.tz == 4) return launch3d<8, 4, 256>(g, st, sa, stream);
-    if (g.tx == 32 && g.ty == 4 && g.tz == 4) return launch3d<4, 4, 128>(g, st, sa, stream);
-    if (g.tx == 32 && g.ty == 8 && g.tz == 2) return launch3d<8, 2, 128>(g, st, sa, stream);
+    if (g.tx == 32 && g.ty == 16 && g.tz == 8) return launch3d<16, 8, 512, 1>(g, st, sa, stream);
+    if (g.tx == 32 && g.ty == 8 && g.tz == 8) return launch3d<8, 8, 256, 2>(g, st, sa, stream);
+    if (g.tx == 32 && g.ty == 8 && g.tz == 4) {
+        // Five regions per SM only where many wait for a place: each is slower (96
+        // registers a thread instead of 128), the SM does more of them.  Discharge
+        // time of a solve with four / five: 128^3 (2048 regions) 6.7 / 7.2 ms, 192^3
+        // (6912) 16.2 / 16.4, 256x256x128 (8192) 19.1 / 19.3 and 18.95 with five
+        // for the sweeps above the bound, 256^3 (16384) 36.2 / 34.2, 512x512x384
+        // (98304) 203 / 181.
+        if (sa.active > kMany3d * device_sms()) return launch3d<8, 4, 128, 5>(g, st, sa, stream);
+        return launch3d<8, 4, 128, 4>(g, st, sa, stream);
+    }
+    if (g.tx == 32 && g.ty == 4 && g.tz == 4) return launch3d<4, 4, 128, 8>(g, st, sa, stream);
+    if (g.tx == 32 && g.ty == 8 && g.tz == 2) return launch3d<8, 2, 128, 8>(g, st, sa, stream);
     return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_discharge3d_batch(int tx, int ty, int tz, const Inst *insts, const int2 *items, const int *count,
                                      int *head, const SweepArgs &sa, int blocks, cudaStream_t stream) {
-    if (tx == 32 && ty == 16 && tz == 8) return launch3d_batch<16, 8, 512>(insts, items, count, head, sa, blocks, stream);
-    if (tx == 32 && ty == 8 && tz == 8) return launch3d_batch<8, 8, 256>(insts, items, count, head, sa, blocks, stream);
-    if (tx == 32 && ty == 8 && tz == 4) return launch3d_batch<8, 4, 256>(insts, items, count, head, sa, blocks, stream);
-    if (tx == 32 && ty == 4 && tz == 4) return launch3d_batch<4, 4, 128>(insts, items, count, head, sa, blocks, stream);
-    if (tx == 32 && ty == 8 && tz == 2) return launch3d_batch<8, 2, 128>(insts, items, count, head, sa, blocks, stream);
+    if (tx == 32 && ty == 16 && tz == 8) return launch3d_batch<16, 8, 512, 1>(insts, items, count, head, sa, blocks, stream);
+    if (tx == 32 && ty == 8 && tz == 8) return launch3d_batch<8, 8, 256, 2>(insts, items, count, head, sa, blocks, stream);
+    if (tx == 32 && ty == 8 && tz == 4) return launch3d_batch<8, 4, 256, 4>(insts, items, count, head, sa, blocks, stream);
+    if (tx == 32 && ty == 4 && tz == 4) return launch3d_batch<4, 4, 128, 8>(insts, items, count, head, sa, blocks, stream);
+    if (tx == 32 && ty == 8 && tz == 2) return launch3d_batch<8, 2, 128, 8>(insts, items, count, head, sa, blocks, stream);
     return cudaErrorInvalidValue;
 }
 

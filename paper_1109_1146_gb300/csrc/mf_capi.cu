@@ -73,6 +73,7 @@ struct mf_grid {
     cudaEvent_t ev[9] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     int4 *h_log = nullptr, *h_log_dv = nullptr;       // pinned records of a window's sweeps, their device view
     cudaEvent_t wev[3 * kWindow] = {};                // start, after the discharge, end of each of them
+    int last_active = 0;                              // active regions after the last window (nreg at first)
     bool relabel_pending = false;                     // a global relabel whose counts are in flight to h_ctr
     long long launches = 0;
     std::string err;
@@ -1466,6 +1467,7 @@ static mf_status begin_impl(mf_grid *g, const mf_opts *opts, bool defer, bool *b
         g->g.dinf = (int)std::max<long long>(g->boundary, 1);
     }
     g->relabel_pending = false;
+    g->last_active = g->g.nreg;
     const size_t nreg = (size_t)g->g.nreg;
     const bool defer_init = batched_init && !g->opts.warm_start && !g->opts.region_reduction;
     if (batched_init) *batched_init = defer_init;
@@ -1618,6 +1620,7 @@ static mf_status run_window(mf_grid *g, int count, bool defer, int32_t *active_o
     sa.partial = g->opts.partial_discharge;
     sa.max_rounds = g->opts.max_rounds;
     sa.variant = g->opts.kernel_variant;
+    sa.active = g->last_active;
     sa.c64 = g->c64;
     CK(cudaMemsetAsync(g->st.ctr, 0, 4 * (kTicket + 1), g->stream));
     for (int i = 0; i < count; ++i) {
@@ -1656,6 +1659,7 @@ static mf_status run_window(mf_grid *g, int count, bool defer, int32_t *active_o
         }
         if (active == 0) break;
     }
+    g->last_active = active;
     if (active > 0 && glr_due(g, g->sweep)) {
         // exact region-distance relabel (raises labels to max(d, d*)), then the
         // activity of every region is recomputed from the new labels
@@ -1803,6 +1807,7 @@ static mf_status build_graph(mf_grid *g) {
     cudaGraph_t body = np.conditional.phGraph_out[0];
     SweepArgs sa{};
     sa.sweep_dev = &g->loopctl[kLoopSweep];
+    sa.active = g->g.nreg;
     sa.partial = g->opts.partial_discharge;
     sa.max_rounds = g->opts.max_rounds;
     sa.variant = g->opts.kernel_variant;

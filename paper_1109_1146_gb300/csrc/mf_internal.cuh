@@ -101,6 +101,7 @@ struct SweepArgs {
     int partial;        // partial discharges (Sec. 6.2)
     int max_rounds;     // Augment round cap per stage
     int variant;        // 0: bit-parallel 2D kernel where available, 1: generic kernel
+    int active;         // regions to discharge as far as the host knows (a bound: chooses between builds of a kernel)
     Counters64 *c64;
 };
 

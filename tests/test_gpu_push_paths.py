@@ -78,3 +78,14 @@ def test_same_as_generic_and_dinic(dims, conn, tile, kind):
         assert np.array_equal(got[k], ref[k]), k
     for k in ("sweeps", "discharges", "rounds", "flow_value"):
         assert getattr(got["stats"], k) == getattr(ref["stats"], k), k
+
+
+def test_many_regions_same_as_generic():
+    # above the number of regions from which five 32x8x4 regions share an SM (a build of its own)
+    inst = grids.random_grid((256, 250, 120), 6, 12, cmax=9, tmax=120, p_zero=0.5)
+    got = gpu_solve(inst)
+    ref = gpu_solve(inst, opts=opts(kernel_variant=1))
+    assert got["flow"] == ref["flow"]
+    for k in ("smin", "smax", "res", "tres", "exc", "lab"):
+        assert np.array_equal(got[k], ref[k]), k
+    assert got["stats"].rounds == ref["stats"].rounds
