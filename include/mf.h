@@ -32,7 +32,8 @@
  *     (the list's first pair swapped so that c = 4 would be the 4-connected
  *     grid) with H = c/2; such grids are solved one by one on 32x32 tiles (or
  *     64x32 / 64x64 at c = 8) with
- *     the generic region discharge (kernel_variant 0 or 1 = ARD, 2 = PRD)
+ *     the region discharge (kernel_variant 0 = ARD, bit-parallel on 32x32
+ *     tiles; 1 = generic ARD, 2 = PRD)
  *     and a global relabel of their own (opts.global_relabel_period), without
  *     warm start, region reduction, boundary relabel, batches or
  *     MF_STATE_HOST;
@@ -83,7 +84,7 @@ typedef struct {
     int32_t global_relabel_period; /* P > 0: exact region-distance relabel after every P-th sweep (2D grids and
                                       3D grids with 32-wide tiles; Sec. 4.1 distance); 0 = off; default 4 */
     int32_t max_rounds;            /* cap on Augment rounds per stage inside one discharge; 0 = default 65536 */
-    int32_t kernel_variant;        /* 0: bit-parallel 2D / 3D discharge where the tile allows (default); 1: generic kernel;
+    int32_t kernel_variant;        /* 0: bit-parallel 2D / 3D / stencil discharge where the tile allows (default); 1: generic kernel;
                                       2: Discharge = PRD (push-relabel region discharge of Sec. 3, exact region-relabel
                                       with unit arc lengths every round): the P-PRD algorithm on the same sweep loop,
                                       labels up to d_inf = n, global gap off, sweep cap 2n^2; for comparison */

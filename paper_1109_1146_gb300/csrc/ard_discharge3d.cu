@@ -169,8 +169,9 @@ __device__ __forceinline__ void send_arcs3(unsigned a, const int (&c)[sizeof...(
 // and 5-6 push layers per discharge).  By all warps, a row per warp with a
 // block barrier per layer and the masks rebuilt after a round, a push layer took
 // 2100-2400 cycles and a BFS layer 320-350, now 1000 and 95.  Discharge time of a
-// solve: 382 -> 181 ms (512x512x384), 12.4 -> 6.7 ms (128^3), 6.1 -> 3.4 ms
-// (61x75x53).  128 threads per 32x8x4 region in single solves (the graph warp
+// solve: 382 -> 178 ms (512x512x384), 12.4 -> 6.5 ms (128^3), 6.1 -> 3.2 ms
+// (61x75x53); of that the search of the next stage in a bit set of the halo labels
+// instead of a pass per stage 181 -> 178, 6.7 -> 6.5 and 3.4 -> 3.2 ms.  128 threads per 32x8x4 region in single solves (the graph warp
 // without register spills: 210 -> 203 ms on 512x512x384), 256 in batches (62
 // against 65 ms for the batch of 48 2D and 16 3D grids).
 template <int TY, int TZ, int NT, int MB>

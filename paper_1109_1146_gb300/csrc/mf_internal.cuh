@@ -100,7 +100,7 @@ struct SweepArgs {
     const int *sweep_dev;  // if set, the sweep index is read here (sweeps inside a CUDA graph)
     int partial;        // partial discharges (Sec. 6.2)
     int max_rounds;     // Augment round cap per stage
-    int variant;        // 0: bit-parallel 2D kernel where available, 1: generic kernel
+    int variant;        // 0: bit-parallel kernel where available, 1: generic kernel
     int active;         // regions to discharge as far as the host knows (a bound: chooses between builds of a kernel)
     Counters64 *c64;
 };
@@ -284,8 +284,8 @@ cudaError_t ensure_smem_attr(const void *kernel, int bytes);
 // launchers (ard_discharge.cu)
 size_t discharge_smem_bytes(int conn, int tx, int ty, int tz);
 bool discharge_supported(int conn, int tx, int ty, int tz);
-// the synthetic stencils of Sec. 7.1 (codes 100 + c), generic kernel, single solves;
-// their exact region-distance relabel (glr_stencil.cu, 32x32 tiles)
+// the synthetic stencils of Sec. 7.1 (codes 100 + c), single solves; their exact
+// region-distance relabel (glr_stencil.cu, 32x32 tiles a warp per region)
 bool stencil_glr_supported(int conn, const Geom &g);
 size_t stencil_glr_scratch_bytes(int conn, const Geom &g);
 cudaError_t stencil_glr(int conn, const Geom &g, const DevState &st, void *scratch, cudaStream_t s);
