@@ -89,3 +89,24 @@ def test_many_regions_same_as_generic():
     for k in ("smin", "smax", "res", "tres", "exc", "lab"):
         assert np.array_equal(got[k], ref[k]), k
     assert got["stats"].rounds == ref["stats"].rounds
+
+
+@pytest.mark.parametrize("Z", [40, 262, 281])
+def test_halo_labels_far_apart(Z):
+    # two columns of regions joined at the top only: the halo of a low region holds labels near 0 (the
+    # sinks beside it) and near twice the height, so the next stage lies past the 64 labels kept as bits
+    X, Y = 64, 8
+    nl = np.zeros((3, Z, Y, X), np.int32)
+    nl[1, :, :Y - 1, :] = 2
+    nl[2, :Z - 1] = 4
+    nl[0, Z - 1, :, :X - 1] = 40
+    cs, ct = np.zeros((Z, Y, X), np.int32), np.zeros((Z, Y, X), np.int32)
+    cs[:6, ::3, 3:32:4] = 5
+    ct[0, :, 32:] = 2
+    inst = GridInstance((X, Y, Z), 6, cs.reshape(-1), ct.reshape(-1), nl.reshape(3, -1))
+    got = gpu_solve(inst, tile=(32, 8, 4))
+    assert_parity(inst, got)
+    ref = gpu_solve(inst, tile=(32, 8, 4), opts=opts(kernel_variant=1))
+    for k in ("res", "tres", "exc", "lab"):
+        assert np.array_equal(got[k], ref[k]), k
+    assert got["stats"].rounds == ref["stats"].rounds
