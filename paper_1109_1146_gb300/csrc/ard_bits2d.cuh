@@ -326,7 +326,10 @@ __device__ __forceinline__ void discharge2d_region(const Geom &g, const DevState
         if (!landed) landed = mbar_wait(mbar, mphase);  // once more (bounded) before giving up
         mphase ^= 1u;
         if (__syncthreads_or(!landed)) {  // never expected: report and leave the region untouched
-            if (tid == 0) atomicExch(&st.ctr[kError], 2);
+            if (tid == 0) {
+                region_not_staged(st, r);
+                atomicExch(&st.ctr[kError], 2);
+            }
             return;
         }
     }

@@ -117,6 +117,14 @@ __device__ __forceinline__ bool region_to_discharge(const DevState &st, int r) {
     return false;
 }
 
+// Region r's planes did not arrive in shared memory: it stays as the sweep found
+// it.  Its flags of the sweep before must not reach the fusion, which would
+// apply that sweep's outflows again, and it stays active.
+__host__ __device__ __forceinline__ void region_not_staged(const DevState &st, int r) {
+    st.disc[r] = 0;
+    st.left_active[r] = 1;
+}
+
 // ---- bulk asynchronous copies (TMA engine, no tensor map) into shared memory
 // A transaction barrier (mbarrier) in shared memory counts the bytes of the
 // copies issued against it; the phase completes when they have all landed.
