@@ -683,9 +683,11 @@ static mf_status cnn_fail(mf_cnn *c, mf_status s, const std::string &m) {
 #define CKC(call)                                                                                  \
     do {                                                                                           \
         cudaError_t e_ = (call);                                                                   \
-        if (e_ != cudaSuccess)                                                                     \
+        if (e_ != cudaSuccess) {                                                                   \
+            cudaGetLastError(); /* reported here: the next launch check must not see it again */   \
             return cnn_fail(c, e_ == cudaErrorMemoryAllocation ? MF_ENOMEM : MF_ECUDA,             \
                             std::string(#call) + ": " + cudaGetErrorString(e_));                   \
+        }                                                                                          \
     } while (0)
 
 static void cnn_free_acts(mf_cnn *c) {
@@ -694,6 +696,7 @@ static void cnn_free_acts(mf_cnn *c) {
     for (auto &d : c->dbuf)
         if (d) { cudaFree(d); d = nullptr; }
     c->cap_pix = 0;
+    c->N = 0;  // the last forward's activations are gone: no backward on them
 }
 
 static mf_status cnn_ensure_infer(mf_cnn *c, int N, int H, int W) {
