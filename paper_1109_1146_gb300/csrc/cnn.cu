@@ -600,16 +600,19 @@ static cudaError_t conv_mma(const void *x, int cin, const __nv_bfloat16 *w, cons
     return cudaGetLastError();
 }
 
-// partial sums of a layer's weight gradients: rows of K floats
+// partial sums of a layer's weight gradients: blocks * RGW rows of K floats
 static int wgrad_blocks() { return device_sms() * 2; }
-constexpr size_t kWgradRow = 32 * 32 * 9 + 32;  // the largest layer's sums
-constexpr int kWgradRows = 4;                   // row groups a block may write
+template <int CIN, int COUT> constexpr size_t kWgradPart = (size_t)WgradCfg<CIN, COUT>::RGW *WgradCfg<CIN, COUT>::K;
+// a block's share of the workspace: the most any layer writes (9248 floats, the
+// 32 -> 32 layers; the narrow last layers write 6936 and 5780 in several row groups)
+constexpr size_t kWgradPartMax = std::max({kWgradPart<6, 32>, kWgradPart<10, 32>, kWgradPart<32, 32>, kWgradPart<32, 6>,
+                                           kWgradPart<32, 10>});
 
 template <int CIN, int COUT>
 static cudaError_t conv_wgrad(const float *x, const float *dy, float *part, float *g, int N, int H, int W,
                               cudaStream_t s) {
     using C = WgradCfg<CIN, COUT>;
-    static_assert(C::K <= kWgradRow && C::RGW <= kWgradRows, "partial sums");
+    static_assert(kWgradPart<CIN, COUT> <= kWgradPartMax, "partial sums");
     auto k = conv3x3_wgrad_kernel<CIN, COUT>;
     const cudaError_t e = ensure_smem_attr((const void *)k, (int)C::smem);
     if (e != cudaSuccess) return e;
@@ -661,7 +664,7 @@ struct mf_cnn {
     size_t nparam = 0;
     float *p = nullptr, *g = nullptr, *m = nullptr, *v = nullptr;  // master params, grads, Adam moments
     __nv_bfloat16 *pb = nullptr;                                   // BF16 copy used by the products
-    float *part = nullptr;                                         // partial weight gradients of a backward pass
+    float *part = nullptr;                                         // partial weight gradients of a backward pass (11 MB)
     float *act[5] = {nullptr, nullptr, nullptr, nullptr, nullptr}; // layer outputs of the last kept forward
     float *dbuf[2] = {nullptr, nullptr};                           // gradient ping-pong buffers
     double *dloss = nullptr;
@@ -710,8 +713,11 @@ static mf_status cnn_ensure_infer(mf_cnn *c, int N, int H, int W) {
     return MF_OK;
 }
 
+// all that a forward and the backward after it write: a backward allocates
+// nothing (it may run while a stream is captured)
 static mf_status cnn_ensure(mf_cnn *c, int N, int H, int W) {
     const size_t pix = (size_t)N * H * W;
+    if (!c->part) CKC(cudaMalloc(&c->part, wgrad_blocks() * kWgradPartMax * 4));
     if (pix <= c->cap_pix) return MF_OK;
     cnn_free_acts(c);
     for (int l = 1; l <= 3; ++l) CKC(cudaMalloc(&c->act[l], pix * c->ch[l] * 4));
@@ -907,7 +913,6 @@ mf_status mf_cnn_zero_grad(mf_cnn *c) {
 mf_status mf_cnn_backward(mf_cnn *c, const float *x, const float *dy) {
     if (!c || !x || !dy || !c->N) return cnn_fail(c, MF_EINVAL, "backward needs the last forward's input and dy");
     const int N = c->N, H = c->H, W = c->W;
-    if (!c->part) CKC(cudaMalloc(&c->part, (size_t)wgrad_blocks() * kWgradRows * kWgradRow * 4));
     // gradient of layer l's output lives in cur, with the layer's ReLU applied
     // (layer 4 has none)
     const float *cur = dy;

@@ -33,3 +33,39 @@ def test_a_forward_that_does_not_fit():
     net.backward(x, dy)
     assert torch.equal(y, want_y)
     np.testing.assert_array_equal(net.get_grads(), want_g)
+
+
+@pytest.mark.parametrize("c", [6, 10])
+def test_first_backward_allocates_nothing(c):
+    # the first backward of a network can be captured in a CUDA graph, and adds the same gradients as a plain one
+    shape = (2, 40, 33)
+    ref, x, dy, y = _net_and_data(c, shape)
+    ref.forward(x, y)
+    ref.backward(x, dy)
+    graph, side = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    net = mf.CNN(channels=c, seed=5, stream=side)
+    side.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(side):
+        net.forward(x, y)
+    side.synchronize()
+    with torch.cuda.graph(graph, stream=side):
+        net.backward(x, dy)
+    graph.replay()
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(net.get_grads(), ref.get_grads())
+
+
+def test_gradient_workspace_holds_what_the_largest_layer_writes():
+    # one more training network takes its activations and the partial sums of 2 blocks per SM, 9248 floats each
+    net, x, dy, y = _net_and_data(6, (1, 8, 8))
+    net.forward(x, y)
+    net.backward(x, dy)
+    torch.cuda.synchronize()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    before = torch.cuda.mem_get_info()[0]
+    other = mf.CNN(channels=6, seed=6)
+    other.forward(x, y)
+    other.backward(x, dy)
+    torch.cuda.synchronize()
+    # (allocations come in blocks of 2 MB: the workspace, parameters, activations, gradients)
+    assert before - torch.cuda.mem_get_info()[0] <= 2 * sms * 9248 * 4 + 4 * (2 << 20)
