@@ -100,11 +100,17 @@ def workload_name(side=SIDE):
 
 
 def kernel_name(conn, tile, batch=False):
+    """The discharge kernel a solve launches, with the template arguments up to the threads per block (single
+    solves on 32x8x4 tiles have two builds of it, for four and for five resident blocks)."""
     tx, ty, tz = tile
-    if conn == 6:
-        nt = 512 if ty * tz >= 128 else 128 if ty * tz == 16 else 256
-        return f"ard_discharge3d{'_batch' if batch else ''}_kernel<{ty},{tz},{nt}>"
-    return f"ard_discharge2d{'_batch' if batch else ''}_kernel<{conn},{tx},{ty},{256 if tx * ty <= 2048 else 512}>"
+    b = "_batch" if batch else ""
+    if conn == 6 and tx == 32 and ty * tz in (16, 32, 64, 128):
+        nt = {16: 128, 32: 256 if batch else 128, 64: 256, 128: 512}[ty * tz]
+        return f"ard_discharge3d{b}_kernel<{ty},{tz},{nt}>"
+    if conn in (4, 8) and tx in (32, 64) and tx * ty in (512, 1024, 2048, 4096):
+        nt = {512: 128, 1024: 256, 2048: 256, 4096: 512}[tx * ty]
+        return f"ard_discharge2d{b}_kernel<{conn},{tx},{ty},{nt}>"
+    return f"ard_discharge_kernel<{conn},{tx},{ty},{tz}>"  # the generic kernel's tiles
 
 
 def make_instance(seed, side=SIDE):
