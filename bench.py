@@ -209,11 +209,16 @@ def measured_peak_hbm():
         return 6800.0, "fallback"
 
 
+def kernel_source(kernel):
+    """The file that holds a discharge kernel's body."""
+    return "ard_discharge3d.cu" if kernel.startswith("ard_discharge3d") else "ard_bits2d.cuh"
+
+
 def committed_traffic(kernel, tile):
     """DRAM bytes per discharged vertex of a discharge kernel from the
     committed ncu summaries (profiles/*.txt lines "bench: key = value"), or
-    None if no summary covers this kernel and tile, or if the kernel's source
-    changed since it was taken."""
+    None if no summary covers this kernel and tile, or if the file that holds
+    the kernel's body changed since it was taken."""
     import glob
     for p in sorted(glob.glob(os.path.join(ROOT, "profiles", "*.txt"))):
         kv = {}
@@ -226,7 +231,9 @@ def committed_traffic(kernel, tile):
             continue
         if kv.get("kernel") != kernel or kv.get("tile") != "x".join(str(t) for t in tile):
             continue
-        src = os.path.join(ROOT, "paper_1109_1146_gb300", "csrc", kv.get("source", ""))
+        if kv.get("source") != kernel_source(kernel):
+            continue
+        src = os.path.join(ROOT, "paper_1109_1146_gb300", "csrc", kv["source"])
         try:
             sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
         except Exception:
@@ -234,10 +241,6 @@ def committed_traffic(kernel, tile):
         if kv.get("kernel_sha256_16") == sha:
             return float(kv["dram_bytes_per_discharged_vertex"])
     return None
-
-
-def kernel_source(conn):
-    return "ard_discharge3d.cu" if conn == 6 else "ard_discharge2d.cu"
 
 
 def roofline_of(stats, insts, tiles, batch):
