@@ -1001,7 +1001,7 @@ __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState
         DIAG_LAP(10);
         DIAG_ADD(11, clock64() - diag_t0);
         DIAG_ADD(12, 1);
-        DIAG_ADD(13, rounds);
+        DIAG_ADD(14, rounds);
         DIAG_FLUSH();
         if (s_flow) atomicAdd(st.flow_t, s_flow);
         st.disc[r] = 1;
