@@ -9,6 +9,18 @@
 #include "ard_bits2d.cuh"
 #include "ard_generic.cuh"
 
+#ifdef MF_DIAG  // this unit's copy of the counters (each unit that includes ard_bits2d.cuh has one)
+extern "C" int mf_diag_paper_read(unsigned long long *out, int reset) {
+    if (cudaDeviceSynchronize() != cudaSuccess) return 1;
+    if (cudaMemcpyFromSymbol(out, mf::mf_diag, sizeof(unsigned long long) * 32) != cudaSuccess) return 2;
+    if (reset) {
+        static const unsigned long long z[32] = {0};
+        if (cudaMemcpyToSymbol(mf::mf_diag, z, sizeof(z)) != cudaSuccess) return 3;
+    }
+    return 0;
+}
+#endif
+
 namespace mf {
 
 // the generic kernel's tiles
