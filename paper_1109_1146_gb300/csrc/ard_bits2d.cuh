@@ -131,10 +131,11 @@ __device__ __forceinline__ int top_bit(u64 m, int other) {
     return m ? x : other;
 }
 // Shared-memory accesses of the push at constant offsets (bytes) from an
-// address.  The stores are predicated instructions: as C++ conditions they
-// became branches, at 23 cycles each and 70 where lanes differ.  The add is
-// always executed (a predicate on it turns into a branch as well), amounts of
-// 0 change nothing.
+// address: predicated stores, and an add that is always executed (an amount of
+// 0 changes nothing).  Timed in one warp: a predicated store 4.6 cycles, an
+// unconditional add 4.3, a predicated add 37, a taken branch 23 and a divergent
+// one 45-70.  The lane-per-row push written with C++ conditions ran a solve's
+// discharge 1.35 times as fast as the push by all warps, this 1.8 times.
 template <int OFF>
 __device__ __forceinline__ void st_if(bool p, unsigned a, int v) {
     asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.shared.u32 [%0+%3], %1;\n}\n" ::"r"(a), "r"(v),
@@ -180,6 +181,9 @@ __device__ __forceinline__ void send_arcs(unsigned a, const int (&c)[sizeof...(D
 // (2048x2048 8-connected, hard seeds), 7.5 -> 4.8 ms (637x419 8-connected).
 // 64 or 128 threads per region instead of 256: 5-20% slower (staging,
 // write-back and crowded layers), also with five or six regions per SM.
+// The masks stay in registers on the 4-connected 32x32 and all 64x32 tiles; the
+// register limits of MINB spill 114 bytes on 8-connected 32x32 tiles, 118 (12) on
+// 32x16 with 8 (4) arcs, 290 on 8-connected 64x64 and 34 at 20 stencil arcs.
 // The stencils of Sec. 7.1 on the same code, against the vertex-by-vertex kernel
 // (ard_generic.cuh): 325 -> 17 ms discharge time of a 500x500 solve at
 // connectivity 8, 60 sweeps.

@@ -1,7 +1,7 @@
 // Region discharge of P-ARD for 3D 6-connected tiles with bit-parallel graph
 // search.
 //
-// The same computation as ard_discharge.cu and ard_discharge2d.cu (Procedure
+// The same computation as ard_discharge.cu and ard_bits2d.cuh (Procedure
 // ARD of Sec. 4.2, Procedure Augment in synchronous rounds of "exact BFS from
 // T_k, then a layered push from the highest BFS layer down", the ARD
 // region-relabel of Sec. 5.1), for tiles 32 voxels wide in x:
@@ -138,8 +138,7 @@ __device__ __forceinline__ int top_bit3(u32 m, int other) {
 // and the planes after the vertex at `a` (the address of its cap[0]) sent dl
 // along arc D; c and rc: the residuals of the arc and of its reverse before.
 // An arc has one writer per step, the excess of its head may have several.
-// (Predicated instructions, and an add that is always executed: as conditions
-// these became branches, see ard_discharge2d.cu.)
+// (Predicated stores and an add that is always executed: timings in ard_bits2d.cuh.)
 template <int OFF>
 __device__ __forceinline__ void st_if3(bool p, unsigned a, int v) {
     asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q st.shared.u32 [%0+%3], %1;\n}\n" ::"r"(a), "r"(v),
@@ -161,7 +160,7 @@ __device__ __forceinline__ void send_arcs3(unsigned a, const int (&c)[sizeof...(
     (send_arc3<TY, V, D>(a, c[D], rc[D], dl[D]), ...);
 }
 
-// One region's discharge, organised as in 2D (ard_discharge2d.cu): the graph
+// One region's discharge, organised as in 2D (ard_bits2d.cuh): the graph
 // warp keeps the masks in registers, runs the searches and pushes the layers
 // by itself, a lane per row; crowded layers, labels to write and the end of
 // the stages are commands to all warps.
@@ -171,9 +170,12 @@ __device__ __forceinline__ void send_arcs3(unsigned a, const int (&c)[sizeof...(
 // 2100-2400 cycles and a BFS layer 320-350, now 1000 and 95.  Discharge time of a
 // solve: 382 -> 178 ms (512x512x384), 12.4 -> 6.5 ms (128^3), 6.1 -> 3.2 ms
 // (61x75x53); of that the search of the next stage in a bit set of the halo labels
-// instead of a pass per stage 181 -> 178, 6.7 -> 6.5 and 3.4 -> 3.2 ms.  128 threads per 32x8x4 region in single solves (the graph warp
-// without register spills: 210 -> 203 ms on 512x512x384), 256 in batches (62
-// against 65 ms for the batch of 48 2D and 16 3D grids).
+// instead of a pass per stage 181 -> 178, 6.7 -> 6.5 and 3.4 -> 3.2 ms.  128 threads
+// per 32x8x4 region in single solves (the graph warp without register spills:
+// 210 -> 203 ms on 512x512x384), 256 in batches (62 against 65 ms for the batch of
+// 48 2D and 16 3D grids, with 46 bytes spilled at 64 registers).  32x8x8 does not
+// spill either; 32x16x8 spills 202 bytes at its 128 registers, 32x4x4 and 32x8x2 94
+// at 64 (eight blocks per SM).
 template <int TY, int TZ, int NT, int MB>
 __device__ __forceinline__ void discharge3d_region(const Geom &g, const DevState &st, const SweepArgs &sa,
                                                    const int r, unsigned long long *mbar, unsigned &mphase) {
@@ -1087,8 +1089,8 @@ cudaError_t launch_discharge3d(const Geom &g, const DevState &st, const SweepArg
     if (g.tx == 32 && g.ty == 16 && g.tz == 8) return launch3d<16, 8, 512, 1>(g, st, sa, stream);
     if (g.tx == 32 && g.ty == 8 && g.tz == 8) return launch3d<8, 8, 256, 2>(g, st, sa, stream);
     if (g.tx == 32 && g.ty == 8 && g.tz == 4) {
-        // Five regions per SM only where many wait for a place: each is slower (96
-        // registers a thread instead of 128), the SM does more of them.  Discharge
+        // Five regions per SM only where many wait for a place: each is slower (95
+        // registers a thread instead of 109), the SM does more of them.  Discharge
         // time of a solve with four / five: 128^3 (2048 regions) 6.7 / 7.2 ms, 192^3
         // (6912) 16.2 / 16.4, 256x256x128 (8192) 19.1 / 19.3 and 18.95 with five
         // for the sweeps above the bound, 256^3 (16384) 36.2 / 34.2, 512x512x384

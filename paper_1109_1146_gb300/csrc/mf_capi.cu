@@ -1,8 +1,9 @@
 // C ABI (include/mf.h) and the non-discharge kernels of the P-ARD sweep:
 //   init      Init of Sec. 2 plus the terminal reduction;
-//   fuse      label and flow fusion of Algorithm 2 on inter-region arcs;
-//   gap_find  global gap of Sec. 5.1 on the histogram of boundary labels;
-//   post      gap application, region activity for the next sweep;
+//   fuse      label and flow fusion of Algorithm 2 on inter-region arcs; its
+//             last block looks for the global gap of Sec. 5.1 on the histogram
+//             of boundary labels (a kernel of its own in batches);
+//   finish    gap application, region activity for the next sweep;
 //   cut       residual closures giving S_min and S_max.
 #include <algorithm>
 #include <climits>
@@ -1807,7 +1808,7 @@ static mf_status build_graph(mf_grid *g) {
     cudaGraph_t body = np.conditional.phGraph_out[0];
     SweepArgs sa{};
     sa.sweep_dev = &g->loopctl[kLoopSweep];
-    sa.active = g->g.nreg;
+    sa.active = g->g.nreg;  // one build for all sweeps of the graph, the one for the grid's region count
     sa.partial = g->opts.partial_discharge;
     sa.max_rounds = g->opts.max_rounds;
     sa.variant = g->opts.kernel_variant;

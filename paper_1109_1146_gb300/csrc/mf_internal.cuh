@@ -68,8 +68,9 @@ struct Geom {
 struct DevState {
     int *cap, *tcap, *exc, *lab, *lab_next, *bout;
     unsigned char *active;       // [nreg] region has active vertices -> discharge next sweep
+    // (single solves keep these two until the next discharge, batches clear them after the sweep)
     unsigned char *disc;         // [nreg] region was discharged in the current sweep
-    unsigned char *left_active;  // [nreg] a discharge left an active vertex (partial discharges)
+    unsigned char *left_active;  // [nreg] 1: the discharge left excess below d_inf; 2: the fusion added some
     unsigned long long *flow_t;  // flow pushed into t by all discharges
     long long *flow0;            // sum of min(cs, ct) (terminal reduction)
     int *hist;                   // [kHistBins + 1] labels of boundary vertices
@@ -86,7 +87,7 @@ enum Ctr : int {
     kStages = 4,         // ARD stages (low 32 bits; also kept in 64-bit below)
     kDischarges = 5,
     kStop = 6,           // an earlier sweep of the window raised an error: discharge nothing
-    kTicket = 7,         // finished blocks of finish_flags_kernel
+    kTicket = 7,         // finished blocks of fuse_warp_kernel, then of finish_sweep_kernel
     kGlrFlags = 8,       // 3 words: global relabel "grew" flags
     kGlrLevels = 11,     // global relabel: levels run
     kCtrWords = 16
@@ -101,7 +102,10 @@ struct SweepArgs {
     int partial;        // partial discharges (Sec. 6.2)
     int max_rounds;     // Augment round cap per stage
     int variant;        // 0: bit-parallel kernel where available, 1: generic kernel
-    int active;         // regions to discharge as far as the host knows (a bound: chooses between builds of a kernel)
+    // Regions to discharge, an estimate that only chooses between builds of a
+    // kernel: the count before the window of sweeps (the fusions in it may
+    // activate more); inside a graph all regions.
+    int active;
     Counters64 *c64;
 };
 
@@ -354,14 +358,14 @@ size_t br_scratch_bytes(const Geom &g, int conn);
 // regions active under the new labels when applied
 cudaError_t boundary_relabel(int conn, const Geom &g, const DevState &st, void *scratch, int *h_words,
                              BrResult *res, cudaStream_t s);
-// ard_discharge2d.cu
+// ard_discharge2d.cu (dispatch), ard_bits2d.cuh (kernel)
 bool discharge2d_supported(int conn, int tx, int ty);
 cudaError_t launch_discharge2d_batch(int conn, int tx, int ty, const Inst *insts, const int2 *items,
                                      const int *count, int *head, const SweepArgs &sa, int blocks,
                                      cudaStream_t stream);
 cudaError_t launch_discharge2d(int conn, const Geom &g, const DevState &st, const SweepArgs &sa,
                                cudaStream_t stream);
-// ard_discharge3d.cu (6-connected, tiles 32x16x8 and 32x8x8)
+// ard_discharge3d.cu (6-connected, tiles 32x16x8, 32x8x8, 32x8x4, 32x4x4 and 32x8x2)
 bool discharge3d_supported(int tx, int ty, int tz);
 cudaError_t launch_discharge3d(const Geom &g, const DevState &st, const SweepArgs &sa, cudaStream_t stream);
 cudaError_t launch_discharge3d_batch(int tx, int ty, int tz, const Inst *insts, const int2 *items, const int *count,
